@@ -178,10 +178,10 @@ int lu_factor_noalloc(int64_t n, double* A, int64_t lda, int32_t* ipiv, const hp
  * then L (unit lower) forward and U backward substitution. trans = 1 solves
  * A^T X = B (U^T, then L^T, then the interchanges in reverse order).
  * B (n x nrhs, ldb) holds b on entry and x on exit. ws (256-byte aligned)
- * must hold lu_solve_workspace_size(n, nrhs) bytes. One right-hand side
- * without transpose runs both triangles in one persistent launch, 64-row
- * diagonal blocks applied through their inverses (the same solution as
- * substitution up to rounding). A zero on the diagonal of U sets
+ * must hold lu_solve_workspace_size(n, nrhs) bytes. Both triangles run in one
+ * persistent launch (several right-hand sides: per batch of columns); for one
+ * right-hand side without transpose 64-row diagonal blocks are applied through
+ * their inverses (the same solution as substitution up to rounding). A zero on the diagonal of U sets
  * info->status = HPL_ERR_SINGULAR (the solve still runs; x has Inf/NaN); a
  * device-side wait that expires sets HPL_ERR_TIMEOUT.
  */
@@ -413,12 +413,13 @@ int hplgb_gemm_config(int what, long long value);
  * block solved in shared memory, the rows below it updated by the DFMA
  * product kernel). Both apply the same fused multiply-adds to every entry in
  * the same order, so the factors are bit-identical.
- * what = 1: lu_solve of one right-hand side (trans = 0) as one persistent
- * launch for both triangles (value 1, the default) or as per-block
- * launches (value 0). The two sum in different orders (the same solution to
- * rounding).
- * what = 2: CTAs of that persistent launch, 0 (default) = one per SM, else
- * at most value (1 .. 4096); the result is the same bits for every value.
+ * what = 1: lu_solve as one persistent launch for both triangles (value 1,
+ * the default; several right-hand sides: one per batch of columns) or as
+ * per-block launches (value 0). The two sum in different orders (the same
+ * solution to rounding).
+ * what = 2: CTAs of that persistent launch, 0 (default) = as many as the SMs
+ * hold, else at most value (1 .. 4096); the result is the same bits for every
+ * value at which the persistent launch fits.
  * Process-wide, not thread-safe; HPL_ERR_INVALID for an unknown switch or
  * value.
  */

@@ -6,10 +6,12 @@
 // blocks), then one CTA per right-hand side applies the blocks in order
 // (reverse order, inverse pairs, for the transposed solve).
 // Triangles, one right-hand side without transpose: both in one persistent
-// launch (k_trsv_wave, below). Otherwise blocked substitution with 64-row
-// diagonal blocks: a diagonal block is solved by one warp per right-hand side
-// with shuffles; the rows below (forward) or above (backward) are then
-// updated by a GEMV/GEMM kernel.
+// launch (k_trsv_wave, below); several right-hand sides or the transposed
+// system: both in one persistent launch per batch of columns (k_trsm_wave).
+// Where neither fits, and by hplgb_lu_config switch 1, blocked substitution
+// with 64-row diagonal blocks: a diagonal block is solved by one warp per
+// right-hand side with shuffles; the rows below (forward) or above (backward)
+// are then updated by a GEMV/GEMM kernel.
 #include <algorithm>
 
 #include "common.cuh"
@@ -141,7 +143,8 @@ __global__ void k_check_udiag(int64_t n, const double* __restrict__ LU, int64_t 
 
 // Workspace: the interchange pairs, then for the one-launch solve of a single
 // right-hand side its published blocks (y, then x: 64 values per row block
-// each) and its abort word.
+// each; the several-column solve keeps its groups' counters there) and the
+// abort word.
 struct SolveWs {
     int* cnt;
     int* dst;
@@ -204,8 +207,8 @@ constexpr int kWaveUEarly = 12;        // CTAs from here on invert their last U 
 constexpr int kInvLd = kTB + 1;
 constexpr unsigned long long kWaveEmpty = ~0ull;   // bit pattern of a block not yet published
 
-int g_solve_wave = 1;                  // single right-hand side: 1 wavefront kernel, 0 per-block launches
-int g_solve_wave_grid = 0;             // CTAs of the wavefront kernel (0: one per SM)
+int g_solve_wave = 1;                  // 1 one-launch kernels, 0 per-block launches
+int g_solve_wave_grid = 0;             // most CTAs of the one-launch kernels (0: what the SMs hold)
 
 __device__ __forceinline__ void ld_relaxed_v2(const double* p, double& a, double& b) {
     asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "l"(p) : "memory");
@@ -609,6 +612,344 @@ static int solve_wave(int64_t n, const double* LU, int64_t lda, double* b, doubl
     return HPL_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Several right-hand sides, or the transposed system: both triangles in one
+// persistent launch. T1 is the lower triangle solved first (L, or U^T when
+// transposed), T2 the upper one solved second (U, or L^T).
+//
+// The right-hand sides are cut into groups of at most W columns; a group is
+// solved by P co-resident CTAs, independently of the other groups. The CTAs of
+// a group own row blocks of 32 round-robin. A block's step: subtract T(q, j)
+// x_j for every block j solved before it, in sweep order, then substitute
+// inside the diagonal block (lane = row, warp = right-hand side, the solved
+// value passed by shuffle; the block's rows are scaled by the reciprocals of
+// its diagonal first, so a step of the substitution is one FMA). Solved blocks
+// go to B; a counter per group and sweep (its front) says how many are there.
+//
+// What bounds it: FP64 issues 2 FMA per clock and SM, so n = 4096 with 64
+// columns is 0.85 ms of FMA per sweep on all SMs, and a single SM takes 2 us
+// per 32 x 32 tile and 8 columns. Hence (a) columns are split over groups, so
+// that a step of the dependent chain (one tile, one substitution, about 1 us
+// of publication) is short; (b) a CTA serves the block it has to finish next
+// as far as the front allows and its later blocks only in the slack; (c) the
+// next tile of both is read into registers ahead of need; (d) 16 warps share
+// an SM, so the barriers of one CTA hide behind another's FMAs. The order of
+// additions into an entry does not depend on the schedule, so neither do the
+// bits. n = 4096 with 64 columns, plain and transposed solve together: 5.3 ms
+// (the FP64 rate allows 3.4), against 52 ms
+// with a diagonal and an update launch per 64 rows, one CTA on the diagonal;
+// with 2 columns a step of the chain costs 5.0 us.
+//
+// Waits are bounded as in k_trsv_wave.
+constexpr int kMb = 32;                 // row block
+constexpr int kMbLd = kMb + 1;
+
+__device__ __forceinline__ int ld_acquire_s32(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed_s32(int* p, int v) {
+    asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// shared memory of k_trsm_wave in doubles: diagonal block, tile, x block,
+// reciprocals, and per owned block the right-hand sides
+__host__ __device__ constexpr size_t msolve_smem_doubles(int W, int R) {
+    return (size_t)2 * kMb * kMbLd + (size_t)W * kMb + kMb + (size_t)R * W * kMb;
+}
+
+template <int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
+k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda, double* B, int64_t ldb, int trans,
+            int G, int P, int width, int* fronts, int* abort_flag, hpl_info* info, int64_t timeout_ns) {
+    constexpr int T = 32 * W, E = kMb * kMb / T;      // threads, tile elements per thread
+    extern __shared__ __align__(16) double msm[];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int g = (int)blockIdx.x % G, p = (int)blockIdx.x / G;
+    const int64_t c0 = (int64_t)g * width;
+    const int ncol = (int)min((int64_t)width, nrhs - c0);
+    const int nblk = (int)((n + kMb - 1) / kMb);
+    const int R = p < nblk ? (nblk - 1 - p) / P + 1 : 0;
+    if (ncol <= 0 || R == 0) return;
+    double* dtile = msm;                              // T(q, q) of the next block, scaled: [column][row]
+    double* tile = dtile + kMb * kMbLd;               // [column][row]
+    double* xs = tile + kMb * kMbLd;                  // [right-hand side][row]
+    double* dinv = xs + W * kMb;
+    double* rhs = dinv + kMb;                         // [owned block][right-hand side][row], own thread only
+    int* nj = (int*)(rhs + (size_t)R * T);            // [owned block] columns subtracted so far
+    int& s_front = nj[R];
+    const uint64_t deadline = globaltimer_ns() + (uint64_t)timeout_ns;
+    const bool live = warp < ncol;
+    double* bcol = B + (c0 + (live ? warp : 0)) * ldb;
+
+    for (int k = 0; k < R; k++) {
+        const int64_t row = (int64_t)(p + k * P) * kMb + lane;
+        rhs[(size_t)k * T + t] = live && row < n ? __ldcg(bcol + row) : 0.0;
+    }
+
+    for (int sweep = 0; sweep < 2; sweep++) {
+        const bool fwd = sweep == 0;
+        const bool unit = fwd != (trans != 0);
+        int* front = fronts + sweep * G + g;
+        // sweep order: position s of the sweep is row block qs(s); owned block
+        // k of the sweep is row block qk(k), its right-hand sides in slot(k)
+        auto qs = [&](int s2) { return fwd ? s2 : nblk - 1 - s2; };
+        auto slot = [&](int k) { return fwd ? k : R - 1 - k; };
+        auto qk = [&](int k) { return p + slot(k) * P; };
+        auto pos = [&](int k) { return fwd ? qk(k) : nblk - 1 - qk(k); };
+        // element e of this thread in the tile T(q, column block j)
+        auto load_tile = [&](int q, int j, double (&v)[E]) {
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                const int hi = warp + W * e;
+                const int64_t r = (int64_t)q * kMb + (trans ? hi : lane), c = (int64_t)j * kMb + (trans ? lane : hi);
+                v[e] = r < n && c < n ? __ldg(LU + (trans ? r * lda + c : c * lda + r)) : 0.0;
+            }
+        };
+        auto store_tile = [&](double* dst, const double (&v)[E]) {
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                const int hi = warp + W * e;
+                dst[trans ? lane * kMbLd + hi : hi * kMbLd + lane] = v[e];
+            }
+        };
+        auto load_x = [&](int j) {
+            const int64_t row = (int64_t)j * kMb + lane;
+            return live && row < n ? __ldcg(bcol + row) : 0.0;
+        };
+        // the diagonal block of row block q, rows scaled by the reciprocals
+        auto load_diag = [&](int q) {
+            const int64_t r = (int64_t)q * kMb + lane;
+            if (warp == 0) dinv[lane] = !unit && r < n ? 1.0 / LU[r * lda + r] : 1.0;
+            double v[E];
+            load_tile(q, q, v);
+            __syncthreads();
+            if (!unit) {
+#pragma unroll
+                for (int e = 0; e < E; e++) v[e] *= dinv[trans ? warp + W * e : lane];
+            }
+            store_tile(dtile, v);
+        };
+
+        for (int k = t; k < R; k += T) nj[k] = 0;
+        if (t == 0) s_front = 0;
+        int kp = 0, jp = 0;                            // block finished next, its next column
+        int ks = R > 1 ? 1 : -1, js = 0;               // the slack's block and column
+        bool xpv = false, xsv = false;                 // x of the column read ahead
+        double pn[E], sn[E], xp = 0.0, xn = 0.0;
+        load_diag(qk(0));
+        if (pos(0) > 0) load_tile(qk(0), qs(0), pn);
+        if (ks > 0) load_tile(qk(ks), qs(0), sn);
+        double acc = rhs[(size_t)slot(0) * T + t];
+        __syncthreads();
+        int f = P == 1 ? nblk : 0;                     // blocks known to be solved (one CTA: its own order)
+
+        auto product = [&](const double (&v)[E], double xv, double a) {
+            store_tile(tile, v);
+            xs[t] = xv;
+            __syncthreads();
+            if (live) {
+                const double* xw = xs + warp * kMb;
+#pragma unroll
+                for (int k = 0; k < kMb; k++) a = fma(-tile[k * kMbLd + lane], xw[k], a);
+            }
+            return a;
+        };
+        for (;;) {
+            if (jp == pos(kp)) {
+                // all columns subtracted: substitution in the diagonal block
+                if (!unit) acc *= dinv[lane];
+                if (live) {
+#pragma unroll
+                    for (int s2 = 0; s2 < kMb; s2++) {
+                        const int j = fwd ? s2 : kMb - 1 - s2;
+                        const double xj = __shfl_sync(0xffffffffu, acc, j);
+                        const double d = dtile[j * kMbLd + lane];
+                        if (fwd ? lane > j : lane < j) acc = fma(-d, xj, acc);
+                    }
+                    const int64_t row = (int64_t)qk(kp) * kMb + lane;
+                    if (row < n) __stcg(bcol + row, acc);
+                }
+                rhs[(size_t)slot(kp) * T + t] = acc;
+                __syncthreads();
+                if (t == 0 && P > 1) {
+                    __threadfence();                   // the barrier and this order every thread's x before the front
+                    st_relaxed_s32(front, pos(kp) + 1);
+                }
+                if (++kp == R) break;
+                if (P > 1) f = max(f, pos(kp - 1) + 1);
+                jp = nj[kp];
+                acc = rhs[(size_t)slot(kp) * T + t];
+                if (jp < pos(kp)) load_tile(qk(kp), qs(jp), pn);
+                xpv = false;
+                load_diag(qk(kp));
+                if (ks == kp) {
+                    ks = kp + 1 < R ? kp + 1 : -1;
+                    if (ks > 0) {
+                        js = nj[ks];
+                        load_tile(qk(ks), qs(js), sn);   // js <= front < pos(ks)
+                        xsv = false;
+                    }
+                }
+                __syncthreads();
+                continue;
+            }
+            int fnew = f;
+            bool ordered = false;                      // the counter was read with acquire
+            if (jp < f) {
+                const int j = jp++;
+                const double xv = xpv ? xp : load_x(qs(j));
+                if (t == 0 && P > 1) fnew = ld_relaxed_s32(front);
+                // product() reads pn before the next tile is fetched into it
+                double v[E];
+#pragma unroll
+                for (int e = 0; e < E; e++) v[e] = pn[e];
+                if (jp < pos(kp)) {
+                    load_tile(qk(kp), qs(jp), pn);
+                    xpv = jp < f;
+                    if (xpv) xp = load_x(qs(jp));
+                }
+                acc = product(v, xv, acc);
+            } else if (ks > 0 && js < f) {
+                const int k = ks, j = js;
+                const double xv = xsv ? xn : load_x(qs(j));
+                if (t == 0 && P > 1) fnew = ld_relaxed_s32(front);
+                double v[E];
+#pragma unroll
+                for (int e = 0; e < E; e++) v[e] = sn[e];
+                // next of the slack: the first later block that can use a solved
+                // column, else the first one with columns left
+                int kn = -1, jn = 0;
+                for (int k2 = kp + 1; k2 < R; k2++) {
+                    const int j2 = k2 == k ? j + 1 : nj[k2];
+                    if (j2 < f) {
+                        kn = k2;
+                        jn = j2;
+                        break;
+                    }
+                    if (kn < 0 && j2 < pos(k2)) {
+                        kn = k2;
+                        jn = j2;
+                    }
+                }
+                if (kn > 0) {
+                    load_tile(qk(kn), qs(jn), sn);
+                    xsv = jn < f;
+                    if (xsv) xn = load_x(qs(jn));
+                }
+                double* a = rhs + (size_t)slot(k) * T + t;
+                *a = product(v, xv, *a);
+                if (t == 0) nj[k] = j + 1;             // read again only after the barrier below
+                ks = kn;
+                js = jn;
+            } else if (t == 0) {
+                // nothing to do until the next block of the sweep is solved
+                ordered = true;
+                for (uint32_t it = 0;; it++) {
+                    fnew = ld_acquire_s32(front);
+                    if (fnew > f) break;
+                    if ((it & 63) == 63) {
+                        if (ld_relaxed_s32(abort_flag)) {
+                            fnew = -1;
+                            break;
+                        }
+                        if (globaltimer_ns() > deadline) {
+                            atomicExch(abort_flag, 1);
+                            if (info) info->status = HPL_ERR_TIMEOUT;
+                            fnew = -1;
+                            break;
+                        }
+                    }
+                }
+            }
+            if (t == 0 && P > 1) {
+                if (fnew > f && !ordered) __threadfence();   // the reads of x come after the counter's
+                s_front = fnew;
+            }
+            __syncthreads();
+            if (P > 1) {
+                f = s_front;
+                if (f < 0) return;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// CTAs of k_trsm_wave<W> the device holds at once with smem bytes each
+// (0: unavailable); raises the kernel's shared-memory limit once per device.
+template <int W>
+static int msolve_ctas(size_t smem, size_t limit) {
+    static std::atomic<int> ready[kMaxDevices];
+    const int dv = device_slot();
+    int per = 0, dev = 0, sms = 0;
+    if (dv < 0 || smem > limit) return 0;
+    const void* f = (const void*)k_trsm_wave<W>;
+    if (!ready[dv].load()) {
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        ready[dv].store(1);
+    }
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, 32 * W, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return std::min(per, 16 / W) * sms;
+}
+
+// Both triangles for nrhs right-hand sides in groups of at most W columns;
+// returns -1 (nothing launched) when the kernel is unavailable or one group's
+// blocks do not fit in the shared memory of all CTAs. flags: 2 * nflags ints.
+template <int W>
+static int solve_multi(int64_t n, int64_t nrhs, const double* LU, int64_t lda, double* B, int64_t ldb, int trans,
+                       int* flags, int64_t nflags, int* abort_flag, hpl_info* info, cudaStream_t s) {
+    const size_t limit = wave_smem_limit();
+    const int64_t nblk = (n + kMb - 1) / kMb;
+    auto bytes = [](int64_t R) { return msolve_smem_doubles(W, (int)R) * sizeof(double) + (size_t)(R + 1) * sizeof(int); };
+    // blocks a CTA may own with 16 / W CTAs on an SM (a KB of each is reserved)
+    const size_t share = limit / (16 / W) - 1024;
+    if (share < bytes(1) || n > (int64_t)1 << 30) return -1;
+    const int64_t rmax = std::min<int64_t>(nblk, (int64_t)((share - bytes(0)) / (bytes(1) - bytes(0))));
+    int64_t C = msolve_ctas<W>(bytes(rmax), limit);
+    if (g_solve_wave_grid > 0) C = std::min<int64_t>(C, g_solve_wave_grid);
+    const int64_t pmin = (nblk + rmax - 1) / rmax;
+    if (C < pmin) return -1;
+    // groups of at most W columns, as even as possible; as many of them per
+    // launch as the CTAs hold
+    const int64_t groups = (nrhs + W - 1) / W;
+    int64_t gb = std::min(groups, C / pmin);
+    const int64_t batches = (groups + gb - 1) / gb;
+    gb = (groups + batches - 1) / batches;
+    int64_t P = std::min(nblk, C / gb);
+    if (P > 1 && gb > nflags) {                       // a tiny system with many columns: no waiting
+        P = 1;
+        if (pmin > 1) return -1;
+    }
+    const int width = (int)((nrhs + groups - 1) / groups);
+    const int64_t R = (nblk + P - 1) / P;
+    int64_t timeout_ns = kDefaultTimeoutNs;
+    HPL_CUDA_TRY(cudaMemsetAsync(abort_flag, 0, sizeof(int), s));
+    for (int64_t g0 = 0; g0 < groups; g0 += gb) {
+        int G = (int)std::min(gb, groups - g0), Pi = (int)P, wi = width;
+        int64_t nr = std::min<int64_t>(nrhs - g0 * width, (int64_t)G * width);
+        if (nr <= 0) break;
+        double* Bg = B + g0 * width * ldb;
+        if (P > 1) HPL_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int) * 2 * (size_t)G, s));
+        void* args[] = {&n, &nr, &LU, &lda, &Bg, &ldb, &trans, &G, &Pi, &wi, &flags, &abort_flag, &info, &timeout_ns};
+        const void* f = (const void*)k_trsm_wave<W>;
+        const dim3 grid((unsigned)(G * Pi)), block(32 * W);
+        if (P > 1) HPL_CUDA_TRY(cudaLaunchCooperativeKernel(f, grid, block, args, bytes(R), s));
+        else HPL_CUDA_TRY(cudaLaunchKernel(f, grid, block, args, bytes(R), s));
+        count_launch();
+    }
+    return HPL_OK;
+}
+
 // One triangle: forward (lower) or backward (upper) blocked substitution.
 static int tri_solve(int64_t n, const double* LU, int64_t lda, int lower, int unit, int trans, double* B, int64_t ldb,
                      int64_t nrhs, cudaStream_t s) {
@@ -660,11 +1001,24 @@ extern "C" int lu_solve(int64_t n, int64_t nrhs, const double* LU, int64_t lda, 
         k_check_udiag<<<(unsigned)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, s>>>(n, LU, lda, info);
         HPL_LAUNCH_CHECK();
     }
+    const bool multi = g_solve_wave && (nrhs > 1 || trans);
+    const int64_t nflags = (n + kTB - 1) / kTB * kTB * 2;      // pairs of ints in w.pub
+    // Group width: with many columns the FMAs bound the solve, and groups of 4
+    // shorten a step of the chain; with few columns or blocks the chain does, and
+    // the wider CTA loads its tiles faster. Measured (ms, width 8 / 4): n = 4096
+    // with 8 columns 1.54 / 1.60, 16: 1.74 / 1.75, 32: 2.01 / 1.94, 64: 2.67 /
+    // 2.60; n = 12000 with 64: 18.7 / 17.7; n = 1001 with 24: 0.417 / 0.430.
+    auto both = [&]() {
+        int* flags = (int*)w.pub;
+        return nrhs > 16 && n >= 2048
+                   ? solve_multi<4>(n, nrhs, LU, lda, B, ldb, trans, flags, nflags, w.abort_flag, info, s)
+                   : solve_multi<8>(n, nrhs, LU, lda, B, ldb, trans, flags, nflags, w.abort_flag, info, s);
+    };
     if (!trans) {
         k_apply_perm<<<(unsigned)nrhs, 512, 0, s>>>(n, nblk, cnt, dst, src, 0, B, ldb);
         HPL_LAUNCH_CHECK();
-        if (nrhs == 1 && g_solve_wave) {
-            int st = solve_wave(n, LU, lda, B, w.pub, w.abort_flag, info, s);
+        if (g_solve_wave) {
+            int st = multi ? both() : solve_wave(n, LU, lda, B, w.pub, w.abort_flag, info, s);
             if (st != -1) return st;
         }
         int st = tri_solve(n, LU, lda, 1, 1, 0, B, ldb, nrhs, s);
@@ -672,9 +1026,11 @@ extern "C" int lu_solve(int64_t n, int64_t nrhs, const double* LU, int64_t lda, 
         st = tri_solve(n, LU, lda, 0, 0, 0, B, ldb, nrhs, s);
         if (st) return st;
     } else {
-        int st = tri_solve(n, LU, lda, 1, 0, 1, B, ldb, nrhs, s);   // U^T z = b
-        if (st) return st;
-        st = tri_solve(n, LU, lda, 0, 1, 1, B, ldb, nrhs, s);       // L^T w = z
+        int st = multi ? both() : -1;
+        if (st == -1) {
+            st = tri_solve(n, LU, lda, 1, 0, 1, B, ldb, nrhs, s);   // U^T z = b
+            if (st == 0) st = tri_solve(n, LU, lda, 0, 1, 1, B, ldb, nrhs, s);       // L^T w = z
+        }
         if (st) return st;
         k_apply_perm<<<(unsigned)nrhs, 512, 0, s>>>(n, nblk, cnt, dst, src, 1, B, ldb);
         HPL_LAUNCH_CHECK();

@@ -437,3 +437,72 @@ def test_lu_solve_wavefront_falls_back_when_a_cta_would_own_too_many_blocks(hpl)
         hpl.lu_config(hpl.LU_SOLVE_WAVE, 1)
     assert launches > 4
     assert torch.equal(b, bl)
+
+
+@pytest.mark.parametrize("trans", [0, 1])
+@pytest.mark.parametrize("n,nrhs", [(1, 2), (31, 8), (32, 9), (33, 17), (96, 3), (257, 65), (1000, 2), (2049, 33)])
+def test_lu_solve_several_columns_matches_oracle(hpl, orc, n, nrhs, trans):
+    """Several right-hand sides (and the transposed system) in one persistent
+    launch: 32-row blocks, groups of 8 columns (4 at n = 2049 with 33), a
+    leading dimension above n. The same bits for every grid size, rows beyond n
+    untouched, and within rounding of the oracle's getrs on the same matrix and
+    of the per-block launches."""
+    import torch
+    A = hpl.generate(6, hpl.STREAM_A, n, n)
+    A0 = _to_np(A).copy(order="F")
+    ipiv, _ = hpl.lu_factor(A, nb=64)
+    B0 = torch.full((nrhs, n + 3), 7.0, dtype=torch.float64, device="cuda")
+    B0[:, :n] = hpl.generate(6, hpl.STREAM_B, n, nrhs).t()
+    outs = []
+    try:
+        for grid in (0, 5, 40):
+            hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, grid)
+            buf = B0.clone()
+            info = hpl.Info()
+            l0 = hpl.launch_count()
+            hpl.lu_solve(A, ipiv, buf.t()[:n], trans=trans, info=info)
+            torch.cuda.synchronize()
+            if grid == 0:        # pairs, zero-pivot check, interchanges, one launch for both triangles
+                assert hpl.launch_count() - l0 == 4
+            assert info.read()["status"] == 0
+            assert (buf[:, n:] == 7.0).all()
+            outs.append(buf)
+        hpl.lu_config(hpl.LU_SOLVE_WAVE, 0)
+        bl = B0.clone()
+        hpl.lu_solve(A, ipiv, bl.t()[:n], trans=trans)
+        torch.cuda.synchronize()
+    finally:
+        hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, 0)
+        hpl.lu_config(hpl.LU_SOLVE_WAVE, 1)
+    for o in outs[1:]:
+        assert torch.equal(o, outs[0])
+    X, Xl = _to_np(outs[0].t()[:n]), _to_np(bl.t()[:n])
+    Xo, _ = orc.solve(A0.T if trans else A0, _to_np(B0.t()[:n]))
+    tol = 100 * n * EPS * max(np.linalg.cond(A0, np.inf), 1.0)
+    assert np.abs(X - Xo).max() / np.abs(Xo).max() <= tol
+    assert np.abs(X - Xl).max() / np.abs(Xo).max() <= tol
+
+
+def test_lu_solve_several_columns_zero_pivot_and_nan_column(hpl):
+    """A zero on U's diagonal sets HPL_ERR_SINGULAR and the solve ends; a NaN in
+    one right-hand side stays in its column."""
+    import torch
+    n = 200
+    A = hpl.generate(8, hpl.STREAM_A, n, n)
+    ipiv, _ = hpl.lu_factor(A, nb=64)
+    B0 = hpl.generate(8, hpl.STREAM_B, n, 5)
+    want = B0.clone()
+    hpl.lu_solve(A, ipiv, want)
+    B = B0.clone()
+    B[n // 2, 2] = float("nan")
+    hpl.lu_solve(A, ipiv, B)
+    torch.cuda.synchronize()
+    keep = [0, 1, 3, 4]
+    assert torch.equal(B[:, keep], want[:, keep]) and torch.isnan(B[:, 2]).all()
+    for trans in (0, 1):
+        S = A.clone()
+        S[150, 150] = 0.0
+        info = hpl.Info()
+        hpl.lu_solve(S, ipiv, B0.clone(), trans=trans, info=info)
+        torch.cuda.synchronize()
+        assert info.read()["status_name"] == "HPL_ERR_SINGULAR"
