@@ -506,3 +506,32 @@ def test_lu_solve_several_columns_zero_pivot_and_nan_column(hpl):
         hpl.lu_solve(S, ipiv, B0.clone(), trans=trans, info=info)
         torch.cuda.synchronize()
         assert info.read()["status_name"] == "HPL_ERR_SINGULAR"
+
+
+@pytest.mark.parametrize("kind", ["uniform", "ties"])
+@pytest.mark.parametrize("n,nb,la", [(2, 64, 0), (31, 32, 0), (33, 64, 1), (65, 64, 0), (129, 40, 1), (513, 64, 0),
+                                     (1100, 256, 1), (1700, 96, 1), (2200, 256, 1), (4300, 128, 1)])
+def test_cluster_leaf_bits(hpl, n, nb, la, kind):
+    """The cluster panel leaf gives the bits of the grid-cooperative one: pivots,
+    factors and the zero-pivot record, from one row per CTA to several hundred,
+    full and ragged widths. "ties": small integers with repeated and zero
+    columns, so that magnitudes tie and pivots vanish."""
+    import torch
+    if kind == "uniform":
+        A0 = hpl.generate(11, hpl.STREAM_A, n, n)
+    else:
+        g = torch.Generator(device="cuda").manual_seed(n)
+        A0 = torch.randint(-2, 3, (n, n), generator=g, device="cuda").to(torch.float64).t()
+        A0[:, n // 2] = A0[:, n // 3]
+        A0[:, n - 1] = 0.0
+    out = []
+    for pfact in (0, 1):
+        A = hpl.colmajor(n, n)
+        A.copy_(A0)
+        ipiv, info = hpl.lu_factor(A, nb=nb, lookahead=la, pfact=pfact)
+        torch.cuda.synchronize()
+        out.append((A, ipiv, info.read()))
+    assert torch.equal(out[0][1], out[1][1])
+    assert torch.equal(out[0][0], out[1][0])
+    assert out[0][2] == out[1][2]
+    assert (out[0][2]["status_name"] == "HPL_OK") == (kind == "uniform")
