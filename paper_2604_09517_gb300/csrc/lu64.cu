@@ -1082,9 +1082,10 @@ __global__ void __launch_bounds__(256) k_emu_combine(int64_t m, int64_t nc, cons
 int launch_gemm_bf16(int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb,
                      float* C, int64_t ldc, int sub, int* err, int64_t timeout_ns, int max_ctas, cudaStream_t s);
 
-// Slices of one step: L21 (m x kb, ld ldl) and the kb x nn block row U12 (ld ldu).
+// Slices of one step: L21 (m x kb, ld ldl; none when m is 0) and the columns
+// col0 .. col0+nn of the block row U12 (U: kb x nn, ld ldu).
 static int emu_slice(const LuWs& w, int64_t m, int64_t nn, int kb, const double* L, int64_t ldl, const double* U,
-                     int64_t ldu, cudaStream_t s) {
+                     int64_t ldu, int64_t col0, cudaStream_t s) {
     const int kbp = (int)emu_kbp(kb);
     const int64_t lds = (int64_t)kEmuSlices * kbp;
     if (m > 0) {
@@ -1092,7 +1093,8 @@ static int emu_slice(const LuWs& w, int64_t m, int64_t nn, int kb, const double*
         HPL_LAUNCH_CHECK();
     }
     if (nn > 0) {
-        k_emu_slice_cols<<<(unsigned)((nn + 7) / 8), 256, 0, s>>>(nn, kb, kbp, U, ldu, (__nv_bfloat16*)w.sB, lds, w.eB);
+        k_emu_slice_cols<<<(unsigned)((nn + 7) / 8), 256, 0, s>>>(nn, kb, kbp, U, ldu, (__nv_bfloat16*)w.sB + col0 * lds,
+                                                                     lds, w.eB + col0);
         HPL_LAUNCH_CHECK();
     }
     return HPL_OK;
@@ -1406,53 +1408,52 @@ extern "C" int lu_factor(int64_t n, double* A, int64_t lda, int32_t* ipiv, const
             HPL_CUDA_TRY(cudaEventRecord(ev_panel, ps));
             HPL_CUDA_TRY(cudaStreamWaitEvent(s, ev_panel, 0));
         }
-        // SWAP on every column outside the panel
-        int64_t ncols_out = c0 + (n - c1);
-        if (ncols_out > 0) {
-            unsigned g = (unsigned)((ncols_out + kSwapCols - 1) / kSwapCols);
+        // SWAP, DTRSM and DGEMM of the trailing columns [x0, x1) (SWAP also of the
+        // finished columns [0, left))
+        auto columns = [&](int64_t x0, int64_t x1, int64_t left) -> int {
+            const int64_t ncols_out = left + (x1 - x0), m2 = n - c1, nx = x1 - x0;
+            int r = HPL_OK;
+            if (ncols_out > 0) {
+                unsigned g = (unsigned)((ncols_out + kSwapCols - 1) / kSwapCols);
+                int slot = phase_begin(s);
+                k_laswp_gather<<<g, 256, 0, s>>>(A, lda, left, x0, x1, w.perm_cnt + par, w.perm_dst + par * 2 * nb,
+                                                 w.perm_src + par * 2 * nb);
+                HPL_LAUNCH_CHECK();
+                // at most 2 kb rows move: read + write of each moved element
+                phase_end(slot, s, PH_SWAP, 2.0 * 2.0 * kb * (double)ncols_out * sizeof(double), (int)k);
+            }
+            if (nx <= 0) return HPL_OK;
             int slot = phase_begin(s);
-            k_laswp_gather<<<g, 256, 0, s>>>(A, lda, c0, c1, n, w.perm_cnt + par, w.perm_dst + par * 2 * nb,
-                                             w.perm_src + par * 2 * nb);
-            HPL_LAUNCH_CHECK();
-            // at most 2 kb rows move: read + write of each moved element
-            phase_end(slot, s, PH_SWAP, 2.0 * 2.0 * kb * (double)ncols_out * sizeof(double), (int)k);
-        }
-        if (c1 < n) {
-            // DTRSM on the block row, then DGEMM: look-ahead columns first
-            const int64_t m2 = n - c1;
-            int slot = phase_begin(s);
-            st = launch_trsm(A, lda, c0, kb, c1, n, s);
-            if (st) return st;
-            phase_end(slot, s, PH_TRSM, (double)kb * (kb - 1) * (double)m2, (int)k);
-            const int64_t la_cols = la ? std::min(nb, n - c1) : n - c1;   // no look-ahead: one update
+            r = launch_trsm(A, lda, c0, kb, x0, x1, s);
+            if (r) return r;
+            phase_end(slot, s, PH_TRSM, (double)kb * (kb - 1) * (double)nx, (int)k);
             slot = phase_begin(s);
             if (emu) {
-                st = emu_slice(w, m2, n - c1, kb, A + c0 * lda + c1, lda, A + c1 * lda + c0, lda, s);
-                if (st) return st;
-                st = emu_update(w, m2, la_cols, kb, 0, A + c1 * lda + c1, lda, w.emu_err, o.timeout_ns, s);
+                // L21 is sliced with the first columns
+                r = emu_slice(w, x0 == c1 ? m2 : 0, nx, kb, A + c0 * lda + c1, lda, A + x0 * lda + c0, lda, x0 - c1, s);
+                if (r) return r;
+                r = emu_update(w, m2, nx, kb, x0 - c1, A + x0 * lda + c1, lda, w.emu_err, o.timeout_ns, s);
             } else {
-                st = launch_dgemm_sub(m2, la_cols, kb, A + c0 * lda + c1, lda, A + c1 * lda + c0, lda,
-                                      A + c1 * lda + c1, lda, s);
+                r = launch_dgemm_sub(m2, nx, kb, A + c0 * lda + c1, lda, A + x0 * lda + c0, lda, A + x0 * lda + c1, lda,
+                                     s);
             }
+            phase_end(slot, s, PH_UPDATE, 2.0 * m2 * nx * kb, (int)k);
+            return r;
+        };
+        // Look-ahead: everything of the next panel's columns first, so that the
+        // next panel starts without the swaps and triangular solve of the rest
+        const int64_t xl = la ? std::min(n, c1 + nb) : c1;
+        if (xl > c1) {
+            st = columns(c1, xl, 0);
             if (st) return st;
-            phase_end(slot, s, PH_UPDATE, 2.0 * m2 * la_cols * kb, (int)k);
-            if (la) {
-                HPL_CUDA_TRY(cudaEventRecord(ev_la, s));
-                HPL_CUDA_TRY(cudaStreamWaitEvent(ps, ev_la, 0));
-                st = panel(k + 1);
-                if (st) return st;
-            }
-            if (n - c1 - la_cols > 0) {
-                slot = phase_begin(s);
-                if (emu)
-                    st = emu_update(w, m2, n - c1 - la_cols, kb, la_cols, A + (c1 + la_cols) * lda + c1, lda,
-                                    w.emu_err, o.timeout_ns, s);
-                else
-                    st = launch_dgemm_sub(m2, n - c1 - la_cols, kb, A + c0 * lda + c1, lda,
-                                          A + (c1 + la_cols) * lda + c0, lda, A + (c1 + la_cols) * lda + c1, lda, s);
-                if (st) return st;
-                phase_end(slot, s, PH_UPDATE, 2.0 * m2 * (n - c1 - la_cols) * kb, (int)k);
-            }
+            HPL_CUDA_TRY(cudaEventRecord(ev_la, s));
+            HPL_CUDA_TRY(cudaStreamWaitEvent(ps, ev_la, 0));
+            st = panel(k + 1);
+            if (st) return st;
+        }
+        st = columns(xl, n, c0);
+        if (st) return st;
+        if (c1 < n) {
             if (!la) {
                 st = panel(k + 1);
                 if (st) return st;
