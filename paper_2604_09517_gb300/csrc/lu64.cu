@@ -668,86 +668,61 @@ __global__ void __launch_bounds__(kLeafClThreads) k_panel_leaf_cl(
 }
 
 // ---------------------------------------------------------------------------
-// SWAP: the sequential interchanges ipiv[k0 .. k0+kb) as a gather. One lane
-// replays them on a list of touched positions (the block's own rows first,
-// then every row beyond the block that a pivot names, found through an
-// open-addressing table in shared memory) and the warp emits (dst, src) pairs
-// with new[dst] = old[src]; the gather kernel then moves whole rows.
+// SWAP: the sequential interchanges ipiv[k0 .. k0+kb) as a gather: (dst, src)
+// pairs with new[dst] = old[src]; the gather kernel then moves whole rows.
 // Block b of the launch handles ipiv[k0_base + b*pb, ... + pb) (clipped at
-// n_end) and writes cnt[b], dst/src + b*2*pb. Shared memory:
-// perm_pairs_smem(pb) bytes.
-// Entries outside [k, n_total) are not interchanges and are skipped.
-__global__ void k_perm_pairs(const int32_t* __restrict__ ipiv, int64_t k0_base, int pb, int64_t n_end,
-                             int64_t n_total, int* __restrict__ cnt, int* __restrict__ dst, int* __restrict__ src) {
-    extern __shared__ int psm[];
-    __shared__ int s_len;
-    const int64_t k0 = k0_base + (int64_t)blockIdx.x * pb;
+// n_end) and writes cnt[b], dst/src + b*2*pb. Entries outside [k, n_total)
+// are not interchanges and are skipped. perm_pairs_threads(pb) threads: one
+// per row that can move (the block's own rows, then the row each pivot names
+// beyond the block, kept by the first pivot that names it), which follows its
+// row back through the interchanges, last to first, to the row it came from.
+// A trace is kb dependent steps of a few integer instructions on pivots read
+// from shared memory, all rows side by side. (Replaying the interchanges in
+// order on one lane cost 0.13 us per pivot: 33 us per 256-pivot block, 11 us
+// per 64, on the panel's critical path, against 9 and 2.9 us now.)
+__global__ void __launch_bounds__(1024) k_perm_pairs(const int32_t* __restrict__ ipiv, int64_t k0_base, int pb,
+                                                     int64_t n_end, int64_t n_total, int* __restrict__ cnt,
+                                                     int* __restrict__ dst, int* __restrict__ src) {
+    extern __shared__ int pv[];   // [pb] the block's pivots, k0 + i where nothing is interchanged
+    __shared__ int s_cnt[32];
+    const int k0 = (int)(k0_base + (int64_t)blockIdx.x * pb);
     const int kb = (int)min((int64_t)pb, n_end - k0);
     cnt += blockIdx.x;
     dst += (int64_t)blockIdx.x * 2 * pb;
     src += (int64_t)blockIdx.x * 2 * pb;
-    const int H = perm_pairs_table(pb);
-    int* pos = psm;               // [2*pb] touched positions
-    int* con = psm + 2 * pb;      // [2*pb] their contents (original row numbers)
-    int* pv = psm + 4 * pb;       // [pb] the block's pivots, read once (coalesced)
-    int* hkey = psm + 5 * pb;     // [H] rows beyond the block seen so far (-1: free)
-    int* hslot = hkey + H;        // [H] their index in pos / con
-    const int lane = threadIdx.x;
-    for (int i = lane; i < kb; i += 32) {
-        pos[i] = (int)(k0 + i);
-        con[i] = (int)(k0 + i);
-        pv[i] = ipiv[k0 + i];
+    const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
+    for (int i = e; i < kb; i += blockDim.x) {
+        const int p = ipiv[k0 + i];
+        pv[i] = p > k0 + i && p < n_total ? p : k0 + i;
     }
-    for (int h = lane; h < H; h += 32) hkey[h] = -1;
-    __syncwarp();
-    if (lane == 0) {
-        int L = kb;
-        for (int i = 0; i < kb; i++) {
-            const int p = pv[i];
-            if (p <= k0 + i || p >= n_total) continue;
-            int q;
-            if (p < k0 + kb) {
-                q = (int)(p - k0);
-            } else {
-                // at most pb rows beyond the block, H >= 2 pb: a free entry always exists
-                for (int h = p & (H - 1);; h = (h + 1) & (H - 1)) {
-                    const int key = hkey[h];
-                    if (key == p) {
-                        q = hslot[h];
-                        break;
-                    }
-                    if (key < 0) {
-                        q = L++;
-                        hkey[h] = p;
-                        hslot[h] = q;
-                        pos[q] = p;
-                        con[q] = p;
-                        break;
-                    }
-                }
-            }
-            const int t = con[i];
-            con[i] = con[q];
-            con[q] = t;
+    __syncthreads();
+    const int own = e - pb;                            // the pivot that names this thread's row (negative: a block row)
+    int to = -1;                                       // the row whose new content is traced
+    if (e < kb) to = k0 + e;
+    else if (own >= 0 && own < kb && pv[own] >= k0 + kb) to = pv[own];
+    int r = to;
+    bool again = false;                                // an earlier pivot names the same row
+    if (to >= 0)
+        for (int i = kb - 1; i >= 0; i--) {
+            const int a = k0 + i, b = pv[i];
+            again = again || (b == to && i < own);
+            r = r == a ? b : r == b ? a : r;
         }
-        s_len = L;
+    const bool mv = to >= 0 && !again && r != to;
+    const unsigned bal = __ballot_sync(0xffffffffu, mv);
+    if (lane == 0) s_cnt[warp] = __popc(bal);
+    __syncthreads();
+    int base = 0, total = 0;
+    for (int q = 0; q < (int)blockDim.x / 32; q++) {
+        if (q < warp) base += s_cnt[q];
+        total += s_cnt[q];
     }
-    __syncwarp();
-    const int L = s_len;
-    // compact the pairs that move something
-    int base_out = 0;
-    for (int b = 0; b < L; b += 32) {
-        int e = b + lane;
-        bool mv = e < L && pos[e] != con[e];
-        unsigned bal = __ballot_sync(0xffffffffu, mv);
-        if (mv) {
-            int o = base_out + __popc(bal & ((1u << lane) - 1));
-            dst[o] = pos[e];
-            src[o] = con[e];
-        }
-        base_out += __popc(bal);
+    if (mv) {
+        const int o = base + __popc(bal & ((1u << lane) - 1));
+        dst[o] = to;
+        src[o] = r;
     }
-    if (lane == 0) *cnt = base_out;
+    if (e == 0) *cnt = total;
 }
 
 // Gather rows for the columns [0, cA) and [cB, n): every CTA takes 8 columns;
@@ -1389,8 +1364,8 @@ extern "C" int lu_factor(int64_t n, double* A, int64_t lda, int32_t* ipiv, const
         int r = panel_rec(n, A, lda, c0, kb, c0, kb, ipiv, w, info, o.timeout_ns, pp, ps);
         if (r) return r;
         int par = (int)(k & 1);
-        k_perm_pairs<<<1, 32, perm_pairs_smem(kb), ps>>>(ipiv, c0, kb, c0 + kb, n, w.perm_cnt + par,
-                                                           w.perm_dst + par * 2 * nb, w.perm_src + par * 2 * nb);
+        k_perm_pairs<<<1, perm_pairs_threads(kb), perm_pairs_smem(kb), ps>>>(
+            ipiv, c0, kb, c0 + kb, n, w.perm_cnt + par, w.perm_dst + par * 2 * nb, w.perm_src + par * 2 * nb);
         HPL_LAUNCH_CHECK();
         // getrf of an m x kb panel: m kb^2 - kb^3/3 flops (leading terms)
         phase_end(slot, ps, PH_PANEL, pm * kb * kb - (double)kb * kb * kb / 3.0, (int)k);

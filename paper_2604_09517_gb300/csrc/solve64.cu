@@ -1,9 +1,9 @@
 // lu_solve: the triangular solves that follow the factorization (paper
 // Sec. III-A.1), FP64.
 //
-// Interchanges: the pivot vector is cut into blocks of 256; one warp per block
-// turns its sequential swaps into (dst, src) pairs (done in parallel for all
-// blocks), then one CTA per right-hand side applies the blocks in order
+// Interchanges: the pivot vector is cut into blocks of 256; one CTA per block
+// turns its sequential swaps into (dst, src) pairs, all blocks side by side,
+// then one CTA per right-hand side applies the blocks in order
 // (reverse order, inverse pairs, for the transposed solve).
 // Triangles, one right-hand side without transpose: both in one persistent
 // launch (k_trsv_wave, below); several right-hand sides or the transposed
@@ -995,7 +995,7 @@ extern "C" int lu_solve(int64_t n, int64_t nrhs, const double* LU, int64_t lda, 
     solve_ws_layout(n, &w, (char*)ws);
     int *cnt = w.cnt, *dst = w.dst, *src = w.src;
     const int nblk = (int)((n + kPivBlock - 1) / kPivBlock);
-    k_perm_pairs<<<nblk, 32, perm_pairs_smem(kPivBlock), s>>>(ipiv, 0, kPivBlock, n, n, cnt, dst, src);
+    k_perm_pairs<<<nblk, perm_pairs_threads(kPivBlock), perm_pairs_smem(kPivBlock), s>>>(ipiv, 0, kPivBlock, n, n, cnt, dst, src);
     HPL_LAUNCH_CHECK();
     if (info) {
         k_check_udiag<<<(unsigned)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, s>>>(n, LU, lda, info);

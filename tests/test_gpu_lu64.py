@@ -535,3 +535,31 @@ def test_cluster_leaf_bits(hpl, n, nb, la, kind):
     assert torch.equal(out[0][0], out[1][0])
     assert out[0][2] == out[1][2]
     assert (out[0][2]["status_name"] == "HPL_OK") == (kind == "uniform")
+
+
+@pytest.mark.parametrize("nb", [1, 31, 64, 250, 512])
+def test_interchange_pairs_give_the_rows_lapack_leaves(hpl, orc, nb):
+    """SWAP of blocks of 1, 31, 64, 250 and 512 pivots, a matrix whose pivots
+    name rows inside the block, beyond it and several times: factors and pivots
+    against the oracle, and the solve's interchanges (blocks of 256) both ways."""
+    import torch
+    n = 600
+    A = hpl.generate(21, hpl.STREAM_A, n, n)
+    # growing rows: the pivot of almost every column is one of the last rows
+    A.mul_(torch.linspace(0.01, 1.0, n, dtype=torch.float64, device="cuda")[:, None])
+    A0 = _to_np(A).copy(order="F")
+    ipiv, info = hpl.lu_factor(A, nb=nb)
+    LUo, ipo, _, gap = orc.getrf(A0)
+    assert gap > 1e-12
+    torch.cuda.synchronize()
+    assert info.read()["status"] == 0
+    assert np.array_equal(_to_np(ipiv), ipo)
+    assert np.abs(_to_np(A) - LUo).max() <= 100 * n * EPS * np.abs(LUo).max()
+    B = hpl.generate(21, hpl.STREAM_B, n, 2)
+    for trans in (0, 1):
+        X = B.clone().t().contiguous().t()
+        hpl.lu_solve(A, ipiv, X, trans=trans)
+        torch.cuda.synchronize()
+        Xo, _ = orc.solve(A0.T if trans else A0, _to_np(B))
+        kappa = np.linalg.cond(A0, np.inf)
+        assert np.abs(_to_np(X) - Xo).max() / np.abs(Xo).max() <= 100 * n * EPS * kappa
