@@ -563,3 +563,27 @@ def test_interchange_pairs_give_the_rows_lapack_leaves(hpl, orc, nb):
         Xo, _ = orc.solve(A0.T if trans else A0, _to_np(B))
         kappa = np.linalg.cond(A0, np.inf)
         assert np.abs(_to_np(X) - Xo).max() / np.abs(Xo).max() <= 100 * n * EPS * kappa
+
+
+@pytest.mark.parametrize("n,nb", [(70, 64), (97, 33), (700, 64), (1300, 200)])
+def test_warp_trsm_bits(hpl, n, nb):
+    """The warp-per-column TRSM (few columns: panels' own and the look-ahead
+    columns, blocks of 1 to 64 rows) gives the bits of the one-kernel TRSM
+    (blocks above 64 by measurement switch) and of a factorization in one
+    panel without any TRSM."""
+    import torch
+    A0 = hpl.generate(13, hpl.STREAM_A, n, n)
+    outs = []
+    try:
+        for blocked, la, width in ((1, 0, nb), (1, 1, nb), (0, 0, nb), (1, 0, min(n, 512))):
+            hpl.lu_config(hpl.LU_TRSM_BLOCKED, blocked)
+            A = hpl.colmajor(n, n)
+            A.copy_(A0)
+            ipiv, info = hpl.lu_factor(A, nb=width, lookahead=la)
+            torch.cuda.synchronize()
+            assert info.read()["status"] == 0
+            outs.append((A, ipiv))
+    finally:
+        hpl.lu_config(hpl.LU_TRSM_BLOCKED, 1)
+    for A, ipiv in outs[1:]:
+        assert torch.equal(A, outs[0][0]) and torch.equal(ipiv, outs[0][1])
