@@ -58,7 +58,17 @@ int launch_generate_dominant_f32(uint64_t seed, int64_t n, void* F, int64_t ldf,
                                  float* A32, cudaStream_t s);
 int launch_residual_vec_t(int64_t n, const double* A, int64_t lda, double* anorm, int norm_mode, const double* x,
                           const double* b, double* r, double* sr, void* ws, cudaStream_t s);
+size_t prod64_ws_bytes(int64_t K, int64_t nn);
+int launch_prod64(int64_t M, int64_t nn, int64_t K, int ta, const double* A, int64_t lda, const double* B, int64_t sk,
+                  int64_t sc, double* C, int64_t ldc, int64_t zstride, int64_t kslice, int split, int neg, void* ws,
+                  int* err, int64_t timeout_ns, cudaStream_t s);
 
+// Smallest order whose block residual and outer product run on the tensor cores
+// (prod64.cu) instead of the DFMA kernels. Forward plus backward of the
+// differentiable solve, DFMA / tensor cores (ms): n = 64 with 4 columns 1.32 /
+// 1.38 (three more launches per product), 130 with 3 1.86 / 1.76, 256 with 64
+// 2.25 / 2.05, 4096 with 64 19.4 / 6.96.
+constexpr int64_t kProd64Min = 128;
 constexpr int kDotBlocks = 304;
 constexpr int kGemvSplitMax = 16;
 // Default panel width: with an FP32 trailing matrix each update step moves 8
@@ -946,8 +956,9 @@ __global__ void __launch_bounds__(256) k_gemvT32(int64_t rows, int64_t cols, con
 
 // ---------------------------------------------------------------------------
 // Several right-hand sides at once: classic refinement on the whole block,
-// with the FP64 residual R = B - op(A) X as one DFMA product split over K and
-// the preconditioner as FP32 block triangular solves with the factor's panels.
+// with the FP64 residual R = B - op(A) X as one product split over K (on the
+// tensor cores at FP64 accuracy, prod64.cu, or DFMA for small orders) and the
+// preconditioner as FP32 block triangular solves with the factor's panels.
 constexpr int kBlkSplit = 4;     // K slices of the block residual
 
 // part[z] (m x nn, ld m) = op(A)(rows, K slice z) X(K slice z, cols), op(A) =
@@ -1262,6 +1273,7 @@ struct MxpWs {
     // GMRES's inner products in FP32 data (opts.inner = FP32; absent otherwise)
     float* A32;        // n x n FP32 copy of A
     double* mvpart;    // kGemvSplitMax x n FP64 chunk sums of A32 z
+    void* p64;         // sliced operand of the tensor-core FP64 products (block refinement)
 };
 
 static size_t mxp_ws_layout(int64_t n, int64_t nb, int m, MxpWs* w, char* base, int64_t nrhs_blk = 0,
@@ -1308,6 +1320,7 @@ static size_t mxp_ws_layout(int64_t n, int64_t nb, int m, MxpWs* w, char* base, 
     // last, so that every offset above (the factor's included) is the same with or without it
     t.A32 = a32 ? (float*)take(sizeof(float) * n * n) : nullptr;
     t.mvpart = a32 ? (double*)take(sizeof(double) * kGemvSplitMax * n) : nullptr;
+    t.p64 = nrhs_blk ? take(std::max(prod64_ws_bytes(n, nrhs_blk), prod64_ws_bytes(nrhs_blk, n))) : nullptr;
     if (w) *w = t;
     return off;
 }
@@ -1853,13 +1866,33 @@ struct Mxp {
     // |b| in w.cmax
     int resid_blk(int64_t k, const double* B, int64_t ldb, const double* X, int64_t ldx) {
         int slot = phase_begin(s);
-        const int64_t kchunk = ((n + kBlkSplit - 1) / kBlkSplit + 15) / 16 * 16;
-        dim3 g((unsigned)((n + 63) / 64), (unsigned)((k + 63) / 64), (unsigned)kBlkSplit);
-        if (trans) k_dgemm_part<true><<<g, 256, 0, s>>>(n, k, n, kchunk, A, lda, X, ldx, w.partb);
-        else k_dgemm_part<false><<<g, 256, 0, s>>>(n, k, n, kchunk, A, lda, X, ldx, w.partb);
-        HPL_LAUNCH_CHECK();
+        int split = kBlkSplit;
+        if (n >= kProd64Min && n <= (int64_t)kBlkSplit * 65536) {
+            // K slices: the fewest that leave the last wave of 128 x 32 tiles
+            // fullest, and at most 65536 k each
+            const int64_t tiles = ((n + 127) / 128) * ((k + 31) / 32);
+            double best = 0.0;
+            for (int z = (int)((n + 65535) / 65536); z <= kBlkSplit && (z == 1 || n >= 256 * z); z++) {
+                const double waves = (double)(tiles * z) / kNumSMsGB300;
+                if (waves / std::ceil(waves) > best + 1e-9) {
+                    best = waves / std::ceil(waves);
+                    split = z;
+                }
+            }
+            const int64_t ks = ((n + split - 1) / split + 15) / 16 * 16;
+            split = (int)((n + ks - 1) / ks);
+            int st = launch_prod64(n, k, n, trans, A, lda, X, 1, ldx, w.partb, n, n * k, ks, split, 0, w.p64, w.err,
+                                   o.timeout_ns, s);
+            if (st) return st;
+        } else {
+            const int64_t kchunk = ((n + kBlkSplit - 1) / kBlkSplit + 15) / 16 * 16;
+            dim3 g((unsigned)((n + 63) / 64), (unsigned)((k + 63) / 64), (unsigned)kBlkSplit);
+            if (trans) k_dgemm_part<true><<<g, 256, 0, s>>>(n, k, n, kchunk, A, lda, X, ldx, w.partb);
+            else k_dgemm_part<false><<<g, 256, 0, s>>>(n, k, n, kchunk, A, lda, X, ldx, w.partb);
+            HPL_LAUNCH_CHECK();
+        }
         HPL_CUDA_TRY(cudaMemsetAsync(w.cmax, 0, sizeof(unsigned long long) * 3 * k, s));
-        k_resid_blk_finish<<<grid_blk(n, k), 256, 0, s>>>(n, k, kBlkSplit, w.partb, B, ldb, w.Rb, n, X, ldx,
+        k_resid_blk_finish<<<grid_blk(n, k), 256, 0, s>>>(n, k, split, w.partb, B, ldb, w.Rb, n, X, ldx,
                                                           w.cmax);
         HPL_LAUNCH_CHECK();
         phase_end(slot, s, PH_RESID, 8.0 * n * n + 2.0 * n * n * (double)k);
@@ -2058,8 +2091,15 @@ static int lu_solve_backward_t(int64_t n, int64_t nrhs, const double* A, int64_t
         dim3 g((unsigned)((n + 63) / 64), (unsigned)((n + 63) / 64));
         if (g.y > 65535) return HPL_ERR_INVALID;
         int slot = phase_begin(s);
-        k_outer_neg<<<g, 256, 0, s>>>(n, nrhs, gradB, ldgb, X, ldx, gradA, ldga);
-        HPL_LAUNCH_CHECK();
+        if (mx.nblk && n >= kProd64Min && nrhs <= 65536) {
+            if ((st = launch_prod64(n, n, nrhs, 0, gradB, ldgb, X, ldx, 1, gradA, ldga, 0, (nrhs + 15) / 16 * 16, 1, 1,
+                                    mx.w.p64, mx.w.err, o.timeout_ns, s)))
+                return st;
+            if ((st = mx.check_err(&worst))) return st;
+        } else {
+            k_outer_neg<<<g, 256, 0, s>>>(n, nrhs, gradB, ldgb, X, ldx, gradA, ldga);
+            HPL_LAUNCH_CHECK();
+        }
         phase_end(slot, s, PH_OTHER, 2.0 * n * n * nrhs);
     } else if (gradA) {
         for (int64_t j = 0; j < n; j++) HPL_CUDA_TRY(cudaMemsetAsync(gradA + j * ldga, 0, sizeof(double) * n, s));
