@@ -8,9 +8,10 @@
 //   kind 0 (general): HPL's LU with partial pivoting in FP64 (Sec. III-A.1):
 //     blocked right-looking, panel factored in SMEM (block argmax with the
 //     first-index tie rule, row swaps, true division, rank-1), interchanges
-//     applied to the other columns, TRSM of the block row, DFMA update of the
-//     trailing matrix in 64 x 64 register-tiled blocks; then P b, forward and
-//     backward substitution.
+//     applied to the other columns, TRSM of the block row, update of the
+//     trailing matrix (panels of 16: on the tensor cores at FP64 accuracy, else
+//     DFMA in 64 x 64 register-tiled blocks); then P b, forward and backward
+//     substitution.
 //   kind 1 (diagonally dominant): the HPL-MxP reading (Sec. III-A.2) used by
 //     mxp_solve, per system: block LU without pivoting of an FP32 copy with
 //     panel width NB, D^-1 by Newton-Schulz with split-BF16 products,
@@ -21,6 +22,7 @@
 // The run launch (queue reset + kernel) holds no host synchronisation, so it
 // can be captured in a CUDA graph and replayed.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <mutex>
@@ -30,6 +32,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace hplgb {
 namespace bt {
@@ -152,8 +155,276 @@ __device__ void upd64(double* A, long long lda, const double* P, int prow, int m
     }
 }
 
+// ---- the same update on the tensor cores, at FP64 accuracy ----
+// C -= L U for a panel of 16 (one k step of an MMA): sliced products as in
+// prod64.cu, with 8 slices of 8 bits in FP16 (exact), because 16 k and 8
+// products of at most 255^2 stay below 2^23, exact in FP32. Index k is scaled by
+// 2^xk, the size of U's row k, and back in L's column k (rows of U of very
+// different sizes, as a badly row-scaled system has them, lose nothing); the
+// slices of row i of L and column j of U hold the 64 bits below its largest
+// entry (2^e(i), 2^e(j)); the products s + t = 2 .. 9 are summed per s + t in tensor
+// memory, combined in 64-bit integers (units 2^-58 of 2^(e(i) + e(j))) and
+// subtracted from C with one FMA. A DFMA update rounds every entry 16 times,
+// this one once, and its FP64 pipe does two operations per entry instead of
+// 16. @UPD@
+// Per 128 rows x 16 columns: the threads cut L (from the panel in shared
+// memory, once per 128 rows) and U (from global memory, fetched two tiles
+// ahead), one thread issues 8 MMAs (slice s of L against slices 1 .. 9 - s of U,
+// N up to 128), and every thread folds 8 entries of one row of the tile before,
+// whose C was fetched while its MMAs ran: two accumulators, two buffers of U.
+// Panels with an infinity, a NaN, a subnormal or an exponent beyond +-400 take
+// upd64.
+constexpr int kTcSlices = 8;
+constexpr int kTcA = kTcSlices * 128 * 16 * 2;       // 32 KB: 128 rows of L
+constexpr int kTcN = 16;                             // columns of a tile
+constexpr int kTcB = kTcSlices * kTcN * 16 * 2;      // 4 KB: a tile's U, two buffers
+constexpr int kTcAcc = kTcSlices * kTcN;             // TMEM columns of an accumulator, two of them
+constexpr int kTcCols = 2 * kTcAcc;
+// Smaller updates take upd64. 304 systems of 64 / 96 / 128 with the line at 16, 32,
+// 64 and 96 rows (ms): 0.254, 0.259, 0.288, 0.285 / 0.435, 0.435, 0.461, 0.547 /
+// 0.648, 0.650, 0.670, 0.757 (before the scales of k).
+constexpr int kTcMinRows = 32;
+struct TcState {
+    uint32_t tmem;
+    uint64_t* bar;          // [2] the MMAs of a tile are done, per accumulator
+    uint32_t tiles;         // tiles so far: the accumulator and its phase
+    uint64_t deadline;
+    volatile int* abort;
+    int* err;
+    unsigned char* As;
+    unsigned char* Bs;
+    short* eL;              // exponents of L's rows (panel rows), U's columns (matrix columns)
+    short* eU;
+    int* xk;                // [16] exponents of U's rows
+};
+
+// exponent e with every |x[k]| 2^(sgn xk) < 2^e; kTcBad outside the path's range
+constexpr int kTcBad = 30000;
+constexpr int kTcZero = -3000;      // xk of a row of zeros
+
+__device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, int sgn) {
+    int mx = -100000;
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < 16; q++) {
+        const int E = tc::expo(x[q]);
+        if (E) mx = max(mx, E + sgn * xk[q]);
+        bad = bad || E == 0x7ff || (E == 0 && x[q] != 0.0);
+    }
+    if (bad) return kTcBad;
+    if (mx < -1000) return 0;       // zeros, or only entries that meet rows of zeros
+    return mx < 1022 - 400 || mx > 1022 + 400 ? kTcBad : mx - 1022;
+}
+
+// The scales of a panel: xk from U's rows, then eL (panel rows prow ..) and eU
+// (columns c1 .. n). Nonzero: this thread met something outside the range. Each
+// thread holds its two columns of U across the reduction (n <= 512). Not
+// inlined, as upd_tc.
+__device__ __noinline__ int tc_levels(const double* A, long long lda, const double* P, int prow, int n, int c1, int k0,
+                                      short* eL, short* eU, int* xk) {
+    static_assert(NMAX <= 2 * THREADS, "two columns per thread");
+    double u[2][16];
+    int bad = 0;
+    if (threadIdx.x < 16) xk[threadIdx.x] = 0;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int c = c1 + threadIdx.x + h * THREADS;
+#pragma unroll
+        for (int q = 0; q < 16; q++) u[h][q] = c < n ? A[(long long)c * lda + k0 + q] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 16; q++) {
+        const int v = __reduce_max_sync(0xffffffffu, max(tc::expo(u[0][q]), tc::expo(u[1][q])));
+        if ((threadIdx.x & 31) == 0) atomicMax(&xk[q], v);
+    }
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        const int v = xk[threadIdx.x];
+        xk[threadIdx.x] = v ? v - 1022 : kTcZero;
+        bad = v && (v < 1022 - 400 || v > 1022 + 400);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int c = c1 + threadIdx.x + h * THREADS;
+        if (c >= n) continue;
+        const int e = tc_level(u[h], xk, -1);
+        bad |= e == kTcBad;
+        eU[c] = (short)e;
+    }
+    for (int r = prow + threadIdx.x; r < n - k0; r += THREADS) {
+        double x[16];
+#pragma unroll
+        for (int q = 0; q < 16; q++) x[q] = P[r * panel_stride<16>() + q];
+        const int e = tc_level(x, xk, 1);
+        bad |= e == kTcBad;
+        eL[r] = (short)e;
+    }
+    return bad;
+}
+
+// one pair of values' digits of slice s (0-based) as two FP16 values: 1024 + d
+// is exact, sgn (1024 + d) - sgn 1024 = sgn d
+struct TcPair {
+    unsigned long long a, b;
+    __half2 sg, off;
+    __device__ __forceinline__ TcPair(double x, double y, int sx, int sy, int e) {
+        a = tc::fixed64(x, sx, e);
+        b = tc::fixed64(y, sy, e);
+        const unsigned s = ((unsigned)__double2hiint(x) >> 31) << 15 | ((unsigned)__double2hiint(y) >> 31) << 31;
+        const unsigned one = 0x3c003c00u | s, big = 0xe400e400u ^ s;
+        sg = *reinterpret_cast<const __half2*>(&one);
+        off = *reinterpret_cast<const __half2*>(&big);
+    }
+    __device__ __forceinline__ unsigned digits(int s) const {
+        const unsigned wa = s < 4 ? (unsigned)(a >> 32) : (unsigned)a, wb = s < 4 ? (unsigned)(b >> 32) : (unsigned)b;
+        const int by = 3 - (s & 3);
+        const unsigned h = (__byte_perm(wa, wb, by | (by + 4) << 8) & 0x00ff00ffu) | 0x64006400u;
+        const __half2 r = __hfma2(*reinterpret_cast<const __half2*>(&h), sg, off);
+        return *reinterpret_cast<const unsigned*>(&r);
+    }
+};
+
+__device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr)
+                 : "memory");
+}
+
+// C (rows r0.., columns c0.., m x m) -= L (panel rows prow..) U (global rows
+// k0.., 16 of them). Returns the new count of tiles; *tc.abort: a wait gave up.
+// Not inlined: its registers stay apart from the other phases' (two CTAs of 256
+// threads share an SM, 128 registers each).
+__device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* P, int prow, int m, long long r0,
+                                        long long c0, long long k0, TcState tc) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row = tid & 127, oct = tid >> 7;                 // cutting L
+    const int bc = tid & 15, kp = (tid >> 4) & 7;              // cutting U (128 threads): column, pair of k
+    const int buf_of = tid >> 7;                               // ... of the tiles with this parity
+    const int frow = (warp & 3) * 32 + lane, half = warp >> 2; // folding: 8 columns of a row
+    const uint32_t as = smem_u32(tc.As), bs = smem_u32(tc.Bs);
+    const int nt = (m + kTcN - 1) / kTcN;
+    for (int ti = 0; ti < m; ti += 128) {
+        {
+            const int r = ti + row;
+            if (r < m) {
+                const double* p = P + (prow + r) * panel_stride<16>() + 8 * oct;
+                const int e = tc.eL[prow + r];
+                const int* x = tc.xk + 8 * oct;
+                const TcPair w[4] = {TcPair(p[0], p[1], x[0], x[1], e), TcPair(p[2], p[3], x[2], x[3], e),
+                                     TcPair(p[4], p[5], x[4], x[5], e), TcPair(p[6], p[7], x[6], x[7], e)};
+                unsigned char* o = tc.As + oct * 2048 + (row >> 3) * 128 + (row & 7) * 16;
+#pragma unroll
+                for (int s = 0; s < kTcSlices; s++)
+                    *reinterpret_cast<uint4*>(o + s * 4096) =
+                        make_uint4(w[0].digits(s), w[1].digits(s), w[2].digits(s), w[3].digits(s));
+            }
+        }
+        double u0 = 0.0, u1 = 0.0;                             // a pair of U of this thread's next tile
+        const int x0 = -tc.xk[2 * kp], x1 = -tc.xk[2 * kp + 1];
+        auto fetch_u = [&](int t) {
+            const int c = t * kTcN + bc;
+            u0 = u1 = 0.0;
+            if (t < nt && c < m) {
+                const double* u = A + (c0 + c) * lda + k0 + 2 * kp;
+                u0 = u[0];
+                u1 = u[1];
+            }
+        };
+        // cut U of tile t (by the threads of its parity) and fetch their next one
+        auto cut_u = [&](int t) {
+            if (t >= nt || buf_of != (t & 1)) return;
+            const int c = t * kTcN + bc, e = c < m ? tc.eU[c0 + c] : 0;
+            const TcPair w(u0, u1, x0, x1, e);
+            unsigned char* o = tc.Bs + (t & 1) * kTcB + (kp >> 2) * (kTcB / 2) + (bc >> 3) * 128 + (bc & 7) * 16 + (kp & 3) * 4;
+#pragma unroll
+            for (int s = 0; s < kTcSlices; s++) *reinterpret_cast<unsigned*>(o + s * (kTcN * 16)) = w.digits(s);
+            fetch_u(t + 2);
+        };
+        fetch_u(buf_of);
+        cut_u(0);
+        const bool rin = ti + frow < m;
+        const int eL = rin ? tc.eL[prow + ti + frow] : 0;
+        double cv[8];
+        double* const crow = A + (c0 + 8 * half) * lda + r0 + ti + frow;
+        auto width = [&](int t) { return rin ? min(8, m - t * kTcN - 8 * half) : 0; };
+        for (int t = 0; t <= nt; t++) {
+            // MMAs of tile t beside the fold of tile t - 1
+            tc::fence_async_smem();
+            tc::tc_fence_before();
+            __syncthreads();
+            if (t > 0) {
+                const int nc = width(t - 1);
+                const double* cp = crow + (long long)(t - 1) * kTcN * lda;
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+                    if (j < nc) cv[j] = cp[j * lda];
+            }
+            if (t < nt) {
+                if (tid == 0) {
+                    tc::tc_fence_after();
+                    const uint32_t d = tc.tmem + ((tc.tiles + t) & 1u) * kTcAcc, b = bs + (t & 1) * kTcB;
+#pragma unroll
+                    for (int q = 0; q < kTcSlices; q++) {
+                        const uint32_t idesc = (1u << 4) | (uint32_t)(kTcN * (kTcSlices - q) >> 3) << 17 | (uint32_t)(128 >> 4) << 24;
+                        const uint64_t ad = tc::desc_plain(as + q * 4096, 2048, 128), bd = tc::desc_plain(b, kTcB / 2, 128);
+                        asm volatile(
+                            "{\n\t.reg .pred p;\n\t"
+                            "setp.ne.b32 p, %4, 0;\n\t"
+                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d + q * kTcN),
+                            "l"(ad), "l"(bd), "r"(idesc), "r"((uint32_t)(q > 0))
+                            : "memory");
+                    }
+                    tc::umma_commit(&tc.bar[(tc.tiles + t) & 1u]);
+                }
+            }
+            if (t == 0) cut_u(1);
+            if (t > 0) {
+                const int f = t - 1;
+                const uint32_t a = (tc.tiles + f) & 1u;
+                const bool ok = tc::mbar_wait(&tc.bar[a], ((tc.tiles + f) >> 1) & 1u, tc.deadline, tc.abort, tc.err);
+                if (!__all_sync(0xffffffffu, ok)) *tc.abort = 1;
+                tc::tc_fence_after();
+                cut_u(t + 1);                              // tile t - 1's slices have been read
+                const uint32_t ta = tc.tmem + ((uint32_t)((warp & 3) * 32) << 16) + a * kTcAcc + half * 8;
+                const int nc = width(f);
+                double* cp = crow + (long long)f * kTcN * lda;
+                const short* eU = tc.eU + c0 + f * kTcN + 8 * half;
+#pragma unroll
+                for (int j4 = 0; j4 < 2; j4++) {
+                    uint32_t g[kTcSlices][4];
+#pragma unroll
+                    for (int q = 0; q < kTcSlices; q++) tc_ld4(ta + q * kTcN + j4 * 4, g[q]);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int jj = j4 * 4 + j;
+                        // neighbours in 32 bits (at most 256 * 7 * 16 * 255^2 + 8 * 16 * 255^2 < 2^31)
+                        auto two = [&](int q) {
+                            return __float2int_rn(__uint_as_float(g[q][j])) * 256 + __float2int_rn(__uint_as_float(g[q + 1][j]));
+                        };
+                        const long long hi = (long long)two(0) * 65536 + two(2);       // units 2^-40
+                        const long long lo = (long long)two(4) * 65536 + two(6);       // units 2^-72
+                        const long long v = hi * (1 << 18) + (lo >> 14);               // units 2^-58
+                        const double scale = __longlong_as_double((long long)(eL + eU[jj] - 58 + 1023) << 52);
+                        if (jj < nc) cp[jj * lda] = fma(-(double)v, scale, cv[jj]);
+                    }
+                }
+            }
+        }
+        tc.tiles += nt;
+        tc::tc_fence_before();
+        __syncthreads();
+        if (*tc.abort) break;
+    }
+    return tc.tiles;
+}
+
+// false: a wait gave up (the system's status is then HPL_ERR_TIMEOUT)
 template <int NB>
-__device__ void lu64(const Sys& S, double* P, double* Us, long long* redk, long long* redi, hpl_info* info) {
+__device__ bool lu64(const Sys& S, double* P, double* Us, long long* redk, long long* redi, hpl_info* info, TcState& tc) {
     __shared__ int s_np, s_dst[2 * NBMAX], s_src[2 * NBMAX], s_pos[2 * NBMAX], s_con[2 * NBMAX];
     const int n = (int)S.n;
     const long long lda = S.lda;
@@ -297,6 +568,8 @@ __device__ void lu64(const Sys& S, double* P, double* Us, long long* redk, long 
         }
         __syncthreads();
         const int c1 = k0 + kb, m = n - c1;
+        int bad = 0;                                     // a row or column of this thread is not for upd_tc
+        const bool use_tc = NB == 16 && kb == 16 && m >= kTcMinRows;
         if (m > 0) {
             // U12 = L11^-1 A12, one thread per column; panels of 16 keep the
             // column's kb entries in registers (same FMAs in the same order)
@@ -328,8 +601,21 @@ __device__ void lu64(const Sys& S, double* P, double* Us, long long* redk, long 
                 for (int i = 1; i < NB; i++)
                     if (i < kb) col[i] = x[i];
             }
-            __syncthreads();
-            upd64<NB>(A, lda, P, kb, m, m, kb, c1, c1, k0, Us);
+            if constexpr (NB == 16)
+                if (use_tc) {
+                    __syncthreads();
+                    bad = tc_levels(A, lda, P, kb, n, c1, k0, tc.eL, tc.eU, tc.xk);
+                }
+            if (use_tc && !__syncthreads_or(bad)) {
+                tc.tiles = upd_tc(A, lda, P, kb, m, c1, c1, k0, tc);
+                if (*tc.abort) {
+                    if (threadIdx.x == 0) info->status = HPL_ERR_TIMEOUT;
+                    return false;
+                }
+            } else {
+                __syncthreads();
+                upd64<NB>(A, lda, P, kb, m, m, kb, c1, c1, k0, Us);
+            }
         }
     }
     __syncthreads();
@@ -400,6 +686,7 @@ __device__ void lu64(const Sys& S, double* P, double* Us, long long* redk, long 
         __syncthreads();
     }
     if (threadIdx.x == 0) info->status = first_zero ? HPL_ERR_SINGULAR : HPL_OK;
+    return true;
 }
 
 // ---- kind 1: BF16 block LU + FP64 refinement ----------------------------------
@@ -673,11 +960,14 @@ __device__ void mxp_one(const Sys& S, const Header* H, float* X, float* R, float
 }
 
 // Dynamic shared memory of a run whose widest panel is NBR: the FP64 panel
-// (NMAX x (NBR + 1)), the U block (NBR x 65), three NBR x NBR FP32 blocks.
+// (NMAX x (NBR + 1)), the U block (NBR x 65; the slices of U for upd_tc), three
+// NBR x NBR FP32 blocks (the exponents for upd_tc), the slices of L.
 template <int NBR>
 constexpr size_t smem_bytes() {
-    return sizeof(double) * (NMAX * panel_stride<NBR>() + NBR * 65) + sizeof(float) * 3 * NBR * NBR;
+    return sizeof(double) * (NMAX * panel_stride<NBR>() + NBR * 65) + sizeof(float) * 3 * NBR * NBR + kTcA;
 }
+static_assert(sizeof(double) * 16 * 65 >= 2 * kTcB && sizeof(float) * 3 * 16 * 16 >= 2 * sizeof(short) * NMAX,
+              "upd_tc's slices of U and exponents share the buffers of the other paths");
 
 }  // namespace bt
 
@@ -903,12 +1193,30 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
     float* R = X + NBR * NBR;
     float* T = R + NBR * NBR;
     __shared__ int s_pref;
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_abort;
+    __shared__ int s_err;
+    __shared__ int s_xk[16];
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kTcCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
     if (threadIdx.x == 0) {
+        tc::mbar_init(&s_bar[0], 1);
+        tc::mbar_init(&s_bar[1], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_abort = 0;
         unsigned smid;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         s_pref = (int)(atomicAdd(&H->sm_slot[smid % kMaxSmSlots], 1u) & 1u);
     }
+    tc::tc_fence_before();
     __syncthreads();
+    tc::tc_fence_after();
+    TcState tc{s_tmem, s_bar, 0u, 0, &s_abort, &s_err, (unsigned char*)(T + NBR * NBR), (unsigned char*)Us, (short*)X,
+               (short*)X + NMAX, s_xk};
     const int pref = s_pref;
     const int lo[2] = {0, H->count0}, sz[2] = {H->count0, H->count - H->count0};
     for (;;) {
@@ -938,12 +1246,15 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
         }
         __syncthreads();
         if (S.kind == 0) {
+            tc.deadline = globaltimer_ns() + (uint64_t)kDefaultTimeoutNs;
+            bool ok;
             if constexpr (NBR == 16) {
-                lu64<16>(S, P, Us, redk, redi, info);
+                ok = lu64<16>(S, P, Us, redk, redi, info, tc);
             } else {
-                if (S.variant) lu64<16>(S, P, Us, redk, redi, info);
-                else lu64<32>(S, P, Us, redk, redi, info);
+                if (S.variant) ok = lu64<16>(S, P, Us, redk, redi, info, tc);
+                else ok = lu64<32>(S, P, Us, redk, redi, info, tc);
             }
+            if (!ok) break;
         } else {
             // the FP64 panel area is free in this path: bf16 operand copies
             if constexpr (NBR == 16) {
@@ -955,6 +1266,21 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
         }
         __syncthreads();
     }
+    if (s_abort && threadIdx.x == 0) {
+        // a wait gave up: the MMAs issued so far end (or have a second) before
+        // TMEM is released
+        __shared__ uint64_t s_drain;
+        tc::mbar_init(&s_drain, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::umma_commit(&s_drain);
+        const uint64_t until = globaltimer_ns() + 1000000000ull;
+        while (!tc::mbar_try_wait(&s_drain, 0) && globaltimer_ns() < until) {}
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(kTcCols) : "memory");
 }
 template __global__ void k_batched_run<NBMAX, 1>(const Sys* __restrict__, Header*, hpl_info*);
 template __global__ void k_batched_run<16, 2>(const Sys* __restrict__, Header*, hpl_info*);

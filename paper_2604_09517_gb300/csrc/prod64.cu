@@ -65,19 +65,6 @@ constexpr int64_t kMaxSlice = 65536;                       // k per CTA: the low
 constexpr int kNoScale = -4000;                            // xk of a zero row of B
 constexpr int kBad = 1 << 24;                              // eB of a column with an infinity or NaN
 
-__device__ __forceinline__ int expo(double v) { return (int)((unsigned)(__double2hiint(v)) >> 20) & 0x7ff; }
-
-// 64-bit fixed point, truncated, of |v| 2^x relative to 2^e (|v| 2^x < 2^e):
-// bit 63 has weight 2^(e-1)
-__device__ __forceinline__ unsigned long long fixed64(double v, int x, int e) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-    const int E = (int)(u >> 52) & 0x7ff;
-    const unsigned long long m = E ? (u << 11) | (1ull << 63) : 0ull;
-    unsigned long long r;
-    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(1022 + e - E - x));    // >= 64: zero
-    return r;
-}
-
 // The 11 slices of 8 consecutive k as 8 BF16 values each (k ascending), handed
 // to put(slice, uint4), from the fixed-point magnitudes T and the signs (bit q
 // of sgn). Digits d < 64 become BF16 through 128 + d (its last place is 1):
@@ -187,13 +174,6 @@ __global__ void __launch_bounds__(256) k_slice_b(int64_t K, int64_t nn, const do
     slices8(T, sgn, [&](int s, uint4 w) { *reinterpret_cast<uint4*>(o + s * (kCols * 16)) = w; });
 }
 
-// Shared-memory descriptor of a K-major tile without swizzle (8 rows x 16
-// bytes core matrices): lead bytes between the two k octets, stride bytes
-// between groups of 8 rows.
-__device__ __forceinline__ uint64_t desc_plain(uint32_t saddr, uint32_t lead, uint32_t stride) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)(lead >> 4) << 16 | (uint64_t)(stride >> 4) << 32 |
-           (uint64_t)1 << 46;
-}
 // kind::f16, BF16 operands, FP32 accumulator, M = 128, N columns
 __device__ __forceinline__ void mma_n(uint32_t d, uint64_t a, uint64_t b, int N, uint32_t accumulate) {
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t)(N >> 3) << 17 | (uint32_t)(kRows >> 4) << 24;

@@ -1,5 +1,6 @@
-// PTX helpers shared by the tensor-core kernels: mbarriers with bounded waits,
-// proxy and tcgen05 fences, commits.
+// Helpers shared by the tensor-core kernels: mbarriers with bounded waits, proxy
+// and tcgen05 fences, commits, operand descriptors, and the fixed-point form of
+// an FP64 value that the sliced products cut up.
 #pragma once
 #include "common.cuh"
 
@@ -55,6 +56,27 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// Shared-memory descriptor of a K-major tile without swizzle (8 rows x 16
+// bytes core matrices): lead bytes between the two k octets, stride bytes
+// between groups of 8 rows.
+__device__ __forceinline__ uint64_t desc_plain(uint32_t saddr, uint32_t lead, uint32_t stride) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)(lead >> 4) << 16 | (uint64_t)(stride >> 4) << 32 |
+           (uint64_t)1 << 46;
+}
+
+__device__ __forceinline__ int expo(double v) { return (int)((unsigned)(__double2hiint(v)) >> 20) & 0x7ff; }
+
+// 64-bit fixed point, truncated, of |v| 2^x relative to 2^e (|v| 2^x < 2^e):
+// bit 63 has weight 2^(e-1)
+__device__ __forceinline__ unsigned long long fixed64(double v, int x, int e) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    const int E = (int)(u >> 52) & 0x7ff;
+    const unsigned long long m = E ? (u << 11) | (1ull << 63) : 0ull;
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(1022 + e - E - x));    // >= 64: zero
+    return r;
+}
 
 }  // namespace tc
 }  // namespace hplgb

@@ -195,3 +195,77 @@ def test_batched_two_ctas_per_sm_same_results(hpl, orc):
     assert out[0][2] == out[1][2]
     with pytest.raises(hpl.HplError):
         hpl.batched_config(1, 0)
+
+
+def _backward_error_bound_holds(A0, LU, piv):
+    """|P A - L U| <= n eps |L| |U| entry by entry (the bound of an LU whose
+    every entry is a sum of rounded products), evaluated in extended precision."""
+    n = A0.shape[0]
+    perm = np.arange(n)
+    for k in range(n):
+        perm[[k, piv[k]]] = perm[[piv[k], k]]
+    L = (np.tril(LU, -1) + np.eye(n)).astype(np.longdouble)
+    U = np.triu(LU).astype(np.longdouble)
+    scale = np.abs(LU).max()
+    R = np.abs(A0[perm].astype(np.longdouble) - L @ U)
+    return bool((R <= n * EPS * (np.abs(L) @ np.abs(U)) + 1e-300 * scale).all())
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+def test_batched_update_backward_error(hpl, orc, variant):
+    """The general systems' factors, with the trailing update on the tensor
+    cores (16-wide panels) and by DFMA (32-wide): entrywise backward error in
+    extended precision at sizes around the update's tiles (16 columns, 128 rows,
+    32 rows as its smallest), pivots equal to the oracle's."""
+    import torch
+    n = np.array([47, 48, 49, 64, 65, 100, 143, 144, 145, 160, 177, 200], dtype=np.int64)
+    bt = hpl.Batch(n, np.zeros(len(n), dtype=np.uint8))
+    bt.generate(23)
+    A0 = [_np(bt.matrix(s)).copy(order="F") for s in range(bt.count)]
+    bt.plan(variant=variant)
+    bt.run()
+    torch.cuda.synchronize()
+    for s in range(bt.count):
+        assert bt.info(s)["status"] == 0
+        piv = _np(bt.pivots(s))
+        _, ipo, _, gap = orc.getrf(A0[s])
+        assert gap > 1e-12 and np.array_equal(piv, ipo)
+        assert _backward_error_bound_holds(A0[s], _np(bt.matrix(s)), piv), int(n[s])
+
+
+def test_batched_update_range(hpl):
+    """Systems outside the tensor-core update's range take DFMA and still meet
+    the bound: entries near 2^600 and 2^-600, subnormal ones, rows and columns
+    of very different sizes; an infinity spreads as in FP64 arithmetic, and the
+    other systems of the batch are untouched."""
+    import torch
+    m = 80
+    n = np.full(7, m, dtype=np.int64)
+    bt = hpl.Batch(n, np.zeros(7, dtype=np.uint8))
+    bt.generate(29)
+    ref = hpl.Batch(n[:1], np.zeros(1, dtype=np.uint8))
+    ref.generate(29)
+    bt.matrix(1).mul_(2.0 ** 600)
+    bt.matrix(2).mul_(2.0 ** -600)
+    bt.matrix(3).mul_(2.0 ** -1030)
+    r = torch.exp2(torch.linspace(-120, 120, m, dtype=torch.float64, device="cuda").round())
+    bt.matrix(4).mul_(r[:, None])
+    bt.matrix(5).mul_(r[None, :])
+    bt.matrix(6)[m - 1, 3] = float("inf")
+    A0 = [_np(bt.matrix(s)).copy(order="F") for s in range(bt.count)]
+    bt.plan(variant=1)
+    ref.plan(variant=1)
+    bt.run()
+    ref.run()
+    torch.cuda.synchronize()
+    assert torch.equal(bt.matrix(0), ref.matrix(0))
+    for s in (0, 1, 2, 4, 5):
+        assert _backward_error_bound_holds(A0[s], _np(bt.matrix(s)), _np(bt.pivots(s))), s
+    piv = _np(bt.pivots(3))          # below 2^-1022 a rounding is absolute: n of them per entry
+    perm = np.arange(m)
+    for k in range(m):
+        perm[[k, piv[k]]] = perm[[piv[k], k]]
+    LU = _np(bt.matrix(3)).astype(np.longdouble)
+    R = np.abs(A0[3][perm] - (np.tril(LU, -1) + np.eye(m)) @ np.triu(LU))
+    assert (R <= m * 2.0 ** -1074 + m * EPS * (np.abs(np.tril(LU, -1) + np.eye(m)) @ np.abs(np.triu(LU)))).all()
+    assert not np.isfinite(_np(bt.matrix(6))).all() and np.isinf(_np(bt.matrix(6))).any()
