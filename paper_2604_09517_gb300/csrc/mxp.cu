@@ -756,8 +756,9 @@ __global__ void __launch_bounds__(256) k_f64_to_bf16_mat2(int64_t n, const doubl
 // Column-split GEMV for the preconditioner: part[s][r] = sum over the column
 // chunk s of P(r, c) x[c]. P is FP32 column-major (rows x cols, ldp); each
 // CTA takes 128 rows (4 per lane, float4 loads when aligned) and one column
-// chunk, its 8 warps split the chunk's columns; k_gemv_combine then adds the
-// chunks in order, so the result does not depend on scheduling.
+// chunk, its 8 warps split the chunk's columns; the last of the CTAs that share
+// the rows (counted in done, left at zero) adds the chunks in order, so the
+// result does not depend on scheduling and takes no further launch.
 __device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float4 ld_f4(const __nv_bfloat16* p) {
     const uint2 u = *reinterpret_cast<const uint2*>(p);
@@ -765,11 +766,29 @@ __device__ __forceinline__ float4 ld_f4(const __nv_bfloat16* p) {
                        __uint_as_float(u.y & 0xffff0000u));
 }
 
+// True in the last of n CTAs to arrive at the counter, which is left at zero;
+// what the others wrote before is then visible (read it with __ldcg).
+__device__ __forceinline__ bool last_cta(unsigned* counter, unsigned n, bool* s_last) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        *s_last = atomicAdd(counter, 1u) == n - 1;
+        if (*s_last) {
+            *counter = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    return *s_last;
+}
+
 template <typename PT>
 __global__ void __launch_bounds__(256) k_gemv_part(int64_t rows, int64_t cols, const PT* __restrict__ P,
                                                    int64_t ldp, const float* __restrict__ x, int64_t chunk,
-                                                   float* __restrict__ part, int64_t ldpart, int vec) {
+                                                   float* part, int64_t ldpart, int vec, unsigned* done,
+                                                   float* y, int sub) {
     __shared__ float red[8][129];
+    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r = (int64_t)blockIdx.x * 128 + 4 * lane;
     const int64_t c0 = (int64_t)blockIdx.y * chunk, c1 = min(cols, c0 + chunk);
@@ -805,14 +824,14 @@ __global__ void __launch_bounds__(256) k_gemv_part(int64_t rows, int64_t cols, c
         for (int w = 0; w < 8; w++) s += red[w][threadIdx.x];
         if (rr < rows) part[blockIdx.y * ldpart + rr] = s;
     }
-}
-
-__global__ void k_gemv_combine(int64_t rows, int nsplit, const float* __restrict__ part, int64_t ldpart,
-                               float* __restrict__ y, int sub) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int q = 0; q < nsplit; q++) s += part[q * ldpart + r];
-        y[r] = sub ? y[r] - s : s;
+    if (!last_cta(done + blockIdx.x, gridDim.y, &s_last)) return;
+    if (threadIdx.x < 128) {
+        const int64_t rr = (int64_t)blockIdx.x * 128 + threadIdx.x;
+        if (rr < rows) {
+            float s = 0.f;
+            for (unsigned q = 0; q < gridDim.y; q++) s += __ldcg(part + q * ldpart + rr);
+            y[rr] = sub ? y[rr] - s : s;
+        }
     }
 }
 
@@ -1216,9 +1235,12 @@ __global__ void k_copy32(int64_t n, const float* __restrict__ a, float* __restri
 }
 
 // --- FP64 vector kernels of the refinement (deterministic reductions) ---
-__global__ void __launch_bounds__(256) k_dot_partial(int64_t n, const double* __restrict__ a,
-                                                     const double* __restrict__ b, double* __restrict__ part) {
+// *out = a . b, or its square root: one partial sum per CTA, added by the last
+// one (counted in done, left at zero) in a fixed order.
+__global__ void __launch_bounds__(256) k_dot(int64_t n, const double* __restrict__ a, const double* __restrict__ b,
+                                             double* part, unsigned* done, double* out, int take_sqrt) {
     __shared__ double sm[256];
+    __shared__ bool s_last;
     double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) s = fma(a[i], b[i], s);
     sm[threadIdx.x] = s;
@@ -1228,12 +1250,9 @@ __global__ void __launch_bounds__(256) k_dot_partial(int64_t n, const double* __
         __syncthreads();
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
-}
-__global__ void __launch_bounds__(256) k_dot_final(int nparts, const double* __restrict__ part, double* out,
-                                                   int take_sqrt) {
-    __shared__ double sm[256];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += 256) s += part[i];
+    if (!last_cta(done, gridDim.x, &s_last)) return;
+    s = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) s += __ldcg(part + i);
     sm[threadIdx.x] = s;
     __syncthreads();
     for (int w = 128; w > 0; w >>= 1) {
@@ -1292,8 +1311,8 @@ struct MxpWs {
     double* part;      // dot partials
     double* scal;      // 4 device scalars (sr, beta, ...)
     float* y32;        // 2n FP32 scratch
-    int* err;          // device error word of the GEMM kernels
-    float* sa;         // n: FP8 / FP16 row scales of a scaled product's A operand
+    int* err;          // device error word of the GEMM kernels; [1] counts the CTAs of k_dot
+    float* sa;         // n: FP8 / FP16 row scales of a scaled product's A operand; in the refinement CTA counters
     float* sb;         // n: FP8 / FP16 column scales of its B operand
     float* gpart;      // kGemvSplitMax x n: column-split GEMV partial sums
     uint64_t* glo;     // kGemvSplitMax x n: exact row-sum partials of a regenerated matrix (low words)
@@ -1412,17 +1431,14 @@ struct Mxp {
         const int64_t chunk = (cols + nsplit - 1) / nsplit;
         nsplit = (cols + chunk - 1) / chunk;
         const int vec = (ldp % 4 == 0) && (((uintptr_t)P & (4 * sizeof(PT) - 1)) == 0);
-        k_gemv_part<<<dim3((unsigned)rb, (unsigned)nsplit), 256, 0, s>>>(rows, cols, P, ldp, x, chunk, w.gpart, n, vec);
-        HPL_LAUNCH_CHECK();
-        k_gemv_combine<<<grid_for(rows), 256, 0, s>>>(rows, (int)nsplit, w.gpart, n, y, sub);
+        k_gemv_part<<<dim3((unsigned)rb, (unsigned)nsplit), 256, 0, s>>>(rows, cols, P, ldp, x, chunk, w.gpart, n, vec,
+                                                                         (unsigned*)w.sa, y, sub);
         HPL_LAUNCH_CHECK();
         return HPL_OK;
     }
 
     int dot(const double* a, const double* b, double* out, int take_sqrt) {
-        k_dot_partial<<<kDotBlocks, 256, 0, s>>>(n, a, b, w.part);
-        HPL_LAUNCH_CHECK();
-        k_dot_final<<<1, 256, 0, s>>>(kDotBlocks, w.part, out, take_sqrt);
+        k_dot<<<kDotBlocks, 256, 0, s>>>(n, a, b, w.part, (unsigned*)w.err + 1, out, take_sqrt);
         HPL_LAUNCH_CHECK();
         return HPL_OK;
     }
@@ -1663,7 +1679,7 @@ struct Mxp {
         if (trans) return precondT(v, out);
         const int64_t ldf = n;
         float* y = w.y32;
-        float* t = w.y32 + n;
+        float* t = w.y32 + n;               // the solution, block by block
         int slot = phase_begin(s);
         k_f64_to_f32<<<grid_for(n), 256, 0, s>>>(n, v, y);
         HPL_LAUNCH_CHECK();
@@ -1677,16 +1693,14 @@ struct Mxp {
         const int64_t last = ((n - 1) / nb) * nb;
         for (int64_t k0 = last; k0 >= 0; k0 -= nb) {
             const int64_t kb = std::min(nb, n - k0);
-            int st = gemv(kb, kb, w.Dinv + k0, n, y + k0, t, 0);
+            int st = gemv(kb, kb, w.Dinv + k0, n, y + k0, t + k0, 0);
             if (st) return st;
-            k_copy32<<<grid_for(kb), 256, 0, s>>>(kb, t, y + k0);
-            HPL_LAUNCH_CHECK();
             if (k0 > 0) {
-                st = gemv(k0, kb, F() + k0 * ldf, ldf, y + k0, y, 1);
+                st = gemv(k0, kb, F() + k0 * ldf, ldf, t + k0, y, 1);
                 if (st) return st;
             }
         }
-        k_f32_to_f64<<<grid_for(n), 256, 0, s>>>(n, y, out);
+        k_f32_to_f64<<<grid_for(n), 256, 0, s>>>(n, t, out);
         HPL_LAUNCH_CHECK();
         phase_end(slot, s, PH_OTHER, 4.0 * n * n + 4.0 * n * nb);
         return HPL_OK;
@@ -1794,6 +1808,9 @@ struct Mxp {
     // Refine one right-hand side. Returns the HPL_* outcome.
     int refine(const double* b, double* x, int* iters, int* inner, double* sr_out, int* status) {
         int rslot = phase_begin(s);
+        // the row counters of the preconditioner's products, in the scales' place
+        // (free once the factorization is done)
+        HPL_CUDA_TRY(cudaMemsetAsync(w.sa, 0, sizeof(float) * n, s));
         int st = refine_body(b, x, iters, inner, sr_out, status);
         phase_end(rslot, s, PH_REFINE, 0.0);
         return st;

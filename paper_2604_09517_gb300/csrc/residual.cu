@@ -200,28 +200,32 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double 
 
 // regen_dominant: the diagonal was skipped by k_res_partial; it is diag[i] if
 // diag is given, else the row's exact sum of |a_ij| rounded once. anorm: a
-// known ||A||_inf (the row sums were not formed), else NULL.
+// known ||A||_inf (the row sums were not formed; diag given), else NULL. rout:
+// receives b - A x if given.
 __global__ void __launch_bounds__(256) k_res_rows(int64_t n, int regen_dominant, const double* __restrict__ diag,
                                                   const double* __restrict__ anorm, const double* __restrict__ x,
-                                                  const double* __restrict__ b, ResWs w) {
+                                                  const double* __restrict__ b, ResWs w, double* __restrict__ rout) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     double mr = 0.0, ma = 0.0, mx = 0.0, mb = 0.0;
     if (i < n) {
         double r = 0.0, s = 0.0;
         uint64_t lo = 0, hi = 0;
-        for (int c = 0; c < kResChunks; c++) {
-            r += w.part_r[c * n + i];
-            s += w.part_a[c * n + i];
-            uint64_t nl = lo + w.part_lo[c * n + i];
-            hi += w.part_hi[c * n + i] + (nl < lo);
-            lo = nl;
+        for (int c = 0; c < kResChunks; c++) r += w.part_r[c * n + i];
+        if (!anorm) {
+            for (int c = 0; c < kResChunks; c++) {
+                s += w.part_a[c * n + i];
+                uint64_t nl = lo + w.part_lo[c * n + i];
+                hi += w.part_hi[c * n + i] + (nl < lo);
+                lo = nl;
+            }
         }
         if (regen_dominant) {
             double d = diag ? diag[i] : res_u128_to_double(hi, lo) * 0x1p-53;
             r = fma(d, x[i], r);
             s += d;
         }
-        r -= b[i];
+        r = b[i] - r;
+        if (rout) rout[i] = r;
         mr = fabs(r);
         ma = anorm ? *anorm : s;
         mx = fabs(x[i]);
@@ -372,11 +376,12 @@ int launch_residual_vec(int64_t n, const double* A, int64_t lda, uint64_t key, c
     dim3 g1((unsigned)((n + 255) / 256), kResChunks);
     k_res_partial<<<g1, 256, 0, s>>>(n, A, lda, key, A ? 0 : 1, dg, x, w, (sr && !anorm) ? 1 : 0);
     HPL_LAUNCH_CHECK();
-    k_res_vec<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, dg, x, b, w, r);
-    HPL_LAUNCH_CHECK();
-    if (sr && b) {
+    if (!(sr && b)) {
+        k_res_vec<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, dg, x, b, w, r);
+        HPL_LAUNCH_CHECK();
+    } else {
         HPL_CUDA_TRY(cudaMemsetAsync(w.maxima, 0, sizeof(unsigned long long) * 4, s));
-        k_res_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, dg != nullptr, dg, anorm, x, b, w);
+        k_res_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, dg != nullptr, dg, anorm, x, b, w, r);
         HPL_LAUNCH_CHECK();
         k_res_final<<<1, 1, 0, s>>>(n, w.maxima, sr);
         HPL_LAUNCH_CHECK();
@@ -395,7 +400,7 @@ int launch_scaled_residual(int64_t n, const double* A, int64_t lda, uint64_t see
     k_res_partial<<<g1, 256, 0, s>>>(n, A, lda, key, kind == HPL_GEN_DIAG_DOMINANT, nullptr, x, w, 2);
     HPL_LAUNCH_CHECK();
     k_res_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, !A && kind == HPL_GEN_DIAG_DOMINANT, nullptr, nullptr,
-                                                           x, b, w);
+                                                           x, b, w, nullptr);
     HPL_LAUNCH_CHECK();
     k_res_final<<<1, 1, 0, s>>>(n, w.maxima, out);
     HPL_LAUNCH_CHECK();
