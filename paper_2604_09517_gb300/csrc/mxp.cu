@@ -1112,19 +1112,29 @@ __global__ void __launch_bounds__(256) k_sgemm(int64_t m, int64_t nn, int64_t kk
     const int64_t row0 = (int64_t)blockIdx.x * 64, col0 = (int64_t)blockIdx.y * 64;
     const int64_t kb0 = (int64_t)blockIdx.z * kslice, kb1 = min(kk, kb0 + kslice);
     float acc[4][4] = {};
+    // the next 16 k are read into registers while the present ones are multiplied
+    float na[4], nb[4];
+    auto fetch = [&](int64_t k0) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int e = tid + 256 * q;
+            const int ka = TA ? e & 15 : e >> 6, r = TA ? e >> 4 : e & 63;
+            const bool oka = k0 + ka < kb1 && row0 + r < m;
+            na[q] = oka ? ld_f(TA ? A + (row0 + r) * lda + k0 + ka : A + (k0 + ka) * lda + row0 + r) : 0.0f;
+            const int c = e >> 4, kb = e & 15;
+            const bool okb = k0 + kb < kb1 && col0 + c < nn;
+            nb[q] = okb ? B[(col0 + c) * ldb + k0 + kb] : 0.0f;
+        }
+    };
+    fetch(kb0);
     for (int64_t k0 = kb0; k0 < kb1; k0 += 16) {
-        for (int e = tid; e < 16 * 64; e += 256) {
-            int kq, r;
-            if (TA) { r = e >> 4; kq = e & 15; }
-            else { kq = e >> 6; r = e & 63; }
-            const bool ok = k0 + kq < kb1 && row0 + r < m;
-            As[kq][r] = ok ? ld_f(TA ? A + (row0 + r) * lda + k0 + kq : A + (k0 + kq) * lda + row0 + r) : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int e = tid + 256 * q;
+            As[TA ? e & 15 : e >> 6][TA ? e >> 4 : e & 63] = na[q];
+            Bs[e & 15][e >> 4] = nb[q];
         }
-        for (int e = tid; e < 16 * 64; e += 256) {
-            const int c = e >> 4, kq = e & 15;
-            const bool ok = k0 + kq < kb1 && col0 + c < nn;
-            Bs[kq][c] = ok ? B[(col0 + c) * ldb + k0 + kq] : 0.0f;
-        }
+        if (k0 + 16 < kb1) fetch(k0 + 16);
         __syncthreads();
 #pragma unroll
         for (int kq = 0; kq < 16; kq++) {
@@ -1970,8 +1980,8 @@ struct Mxp {
             if ((st = resid(B, B, w.r, w.scal))) return st;
         }
         if ((st = read_scalar(w.scal + (trans ? 7 : 6), &anorm))) return st;
-        for (int64_t c = 0; c < k; c++)
-            HPL_CUDA_TRY(cudaMemcpyAsync(w.Rb + c * n, B + c * ldb, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        HPL_CUDA_TRY(cudaMemcpy2DAsync(w.Rb, sizeof(double) * n, B, sizeof(double) * ldb, sizeof(double) * n, (size_t)k,
+                                       cudaMemcpyDeviceToDevice, s));
         if ((st = precond_blk(k, X, ldx, 0))) return st;
         std::vector<unsigned long long> cm((size_t)(3 * k));
         int it = 0;
