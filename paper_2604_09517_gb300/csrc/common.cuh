@@ -136,7 +136,7 @@ __device__ __forceinline__ long long ld_cluster_s64(uint32_t caddr) {
 // output h, built with integer operations only: FP64 conversions and
 // arithmetic issue at the FP64 rate, which is scarce on this part.
 // t = (h >> 11) - 2^52 is the value in units of 2^-53, |t| <= 2^52.
-__device__ __forceinline__ double gen_value(uint64_t h) {
+__device__ __forceinline__ double gen_value_any(uint64_t h) {
     const long long t = (long long)(h >> 11) - (1LL << 52);
     if (t == 0) return 0.0;
     const unsigned long long u = t < 0 ? (unsigned long long)(-t) : (unsigned long long)t;
@@ -145,6 +145,26 @@ __device__ __forceinline__ double gen_value(uint64_t h) {
     const unsigned long long bits =
         ((unsigned long long)(t < 0) << 63) | ((unsigned long long)(p - 53 + 1023) << 52) | mant;
     return __longlong_as_double((long long)bits);
+}
+// The same where top, the upper half of |t| 2^11, is not 0 (the caller looks at
+// it: 0 comes once in 2^31 words): 32-bit operations, the sign taken out with a
+// mask, one shift by the upper half's leading zeros, the leading one carried
+// into the exponent by an addition.
+__device__ __forceinline__ double gen_value_top(uint64_t h, unsigned& top) {
+    const unsigned lo = (unsigned)h, hi = (unsigned)(h >> 32);
+    const unsigned m = ~(unsigned)((int)hi >> 31);             // all ones: t < 0
+    const uint64_t u = ((uint64_t)(hi ^ 0x80000000u ^ m) << 32 | ((lo & 0xfffff800u) ^ m)) - (uint64_t)(int64_t)(int)m;
+    const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
+    top = uh;
+    const int s = __clz((int)uh);
+    const unsigned nh = __funnelshift_l(ul, uh, s), nl = ul << (s & 31);
+    const unsigned e = (m & 0x80000000u) | 0x3fd00000u;        // sign, exponent 1021 (the leading one adds 1)
+    return __hiloint2double((int)(e - ((unsigned)s << 20) + (nh >> 11)), (int)__funnelshift_r(nl, nh, 11));
+}
+__device__ __forceinline__ double gen_value(uint64_t h) {
+    unsigned top;
+    const double a = gen_value_top(h, top);
+    return top ? a : gen_value_any(h);
 }
 
 // Magnitude key of a double for the pivot search: for |v| not NaN the IEEE

@@ -3,7 +3,7 @@
 // formula). A is read, or regenerated from the seed (hpl_generate's
 // definition) so that very large systems need not keep a copy of A.
 //
-// Pass 1: grid (row blocks of 256, column chunks); each thread owns one row
+// Pass 1: grid (row blocks, column chunks); each thread owns one row
 // and sums a_ij x_j and |a_ij| over its chunk (deterministic per-chunk
 // partials). Pass 2: per row, the chunks are summed in order, b_i is
 // subtracted and the maxima are combined with an integer atomicMax on the bit
@@ -15,9 +15,6 @@
 namespace hplgb {
 
 constexpr int kResChunks = 16;
-#ifndef HPLGB_REGEN_I2F
-#define HPLGB_REGEN_I2F 1
-#endif
 
 __host__ __device__ __forceinline__ uint64_t res_mix(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -76,15 +73,68 @@ __device__ __forceinline__ float abs_as_float(double a) {
     return __int_as_float((e << 23) | (int)((u >> 29) & 0x7fffff));
 }
 
-// want_norm: 0 skips the row sums of |a_ij| (plain matrix-vector product),
+// A stored. NORM: 0 skips the row sums of |a_ij| (plain matrix-vector product),
 // 1 sums them in FP32 from abs_as_float (the refinement's stopping test),
-// 2 sums them in FP64 (the HPL acceptance check).
-// A == NULL regenerates the entries from key (hpl_generate's definition); for
-// the dominant matrix the diagonal is skipped here and added per row later,
-// either from the exact row sums accumulated here (diag == NULL) or from diag.
-__global__ void __launch_bounds__(256) k_res_partial(int64_t n, const double* __restrict__ A, int64_t lda,
-                                                     uint64_t key, int dominant, const double* __restrict__ diag,
-                                                     const double* __restrict__ x, ResWs w, int want_norm) {
+// 2 sums them in FP64 (the HPL acceptance check). The product alone is within
+// 10 % of the FP64 pipe's time (n = 16384: 471 us, 426 at two FMA a clock and SM;
+// 321 for reading A). A warp per block: all blocks are resident at once up to
+// n = 9700 and the SMs' shares differ least (32 / 64 / 256 rows per block: n =
+// 4096 43 / 54 / 60 us, 8192 125 / 126 / 144, 16384 471 / 477 / 514, 49152 4025 /
+// 4055 / 4153); four pairs of columns in flight (two: 16384 567 us; eight gain 1 to
+// 5 % above 20000 rows and lose up to 8 % below).
+constexpr int kStoredRows = 32;
+constexpr int kStoredUnroll = 4;      // pairs of columns in flight
+template <int NORM>
+__global__ void __launch_bounds__(kStoredRows) k_res_stored(int64_t n, const double* __restrict__ A, int64_t lda,
+                                                    const double* __restrict__ x, ResWs w) {
+    const int64_t i = (int64_t)blockIdx.x * kStoredRows + threadIdx.x;
+    const int chunk = blockIdx.y;
+    const int64_t cw = (n + kResChunks - 1) / kResChunks;
+    const int64_t j0 = chunk * cw, j1 = std::min<int64_t>(n, j0 + cw);
+    if (i >= n) return;
+    double r = 0.0, s = 0.0;
+    if (NORM == 2) {
+#pragma unroll 8
+        for (int64_t j = j0; j < j1; j++) {
+            double a = A[j * lda + i];
+            r = fma(a, x[j], r);
+            s += fabs(a);
+        }
+    } else {
+        // two interleaved FP64 accumulators shorten the dependent FMA chain
+        double r1 = 0.0;
+        float sf = 0.0f;
+        int64_t j = j0;
+#pragma unroll kStoredUnroll
+        for (; j + 1 < j1; j += 2) {
+            double a0 = A[j * lda + i], a1 = A[(j + 1) * lda + i];
+            r = fma(a0, x[j], r);
+            r1 = fma(a1, x[j + 1], r1);
+            if (NORM) sf += abs_as_float(a0) + abs_as_float(a1);
+        }
+        if (j < j1) {
+            double a0 = A[j * lda + i];
+            r = fma(a0, x[j], r);
+            if (NORM) sf += abs_as_float(a0);
+        }
+        s = (double)sf;
+        r += r1;
+    }
+    w.part_r[chunk * n + i] = r;
+    if (NORM) {
+        w.part_a[chunk * n + i] = s;
+        w.part_lo[chunk * n + i] = 0;
+        w.part_hi[chunk * n + i] = 0;
+    }
+}
+
+// The entries regenerated from key (hpl_generate's definition), with their row
+// sums (want_norm as NORM above, 1 or 2); for the dominant matrix the diagonal
+// is skipped here and added per row later, either from the exact row sums
+// accumulated here (diag == NULL) or from diag.
+__global__ void __launch_bounds__(256) k_res_partial(int64_t n, uint64_t key, int dominant,
+                                                     const double* __restrict__ diag, const double* __restrict__ x,
+                                                     ResWs w, int want_norm) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int chunk = blockIdx.y;
     const int64_t cw = (n + kResChunks - 1) / kResChunks;
@@ -92,64 +142,7 @@ __global__ void __launch_bounds__(256) k_res_partial(int64_t n, const double* __
     if (i >= n) return;
     double r = 0.0, s = 0.0;
     uint64_t lo = 0, hi = 0;
-    if (A) {
-        float sf = 0.0f;
-        if (want_norm == 2) {
-#pragma unroll 8
-            for (int64_t j = j0; j < j1; j++) {
-                double a = A[j * lda + i];
-                r = fma(a, x[j], r);
-                s += fabs(a);
-            }
-        } else {
-            // two interleaved FP64 accumulators shorten the dependent FMA chain
-            double r1 = 0.0;
-            int64_t j = j0;
-            if (want_norm == 1) {
-#pragma unroll 4
-                for (; j + 1 < j1; j += 2) {
-                    double a0 = A[j * lda + i], a1 = A[(j + 1) * lda + i];
-                    r = fma(a0, x[j], r);
-                    r1 = fma(a1, x[j + 1], r1);
-                    sf += abs_as_float(a0) + abs_as_float(a1);
-                }
-                if (j < j1) {
-                    double a0 = A[j * lda + i];
-                    r = fma(a0, x[j], r);
-                    sf += abs_as_float(a0);
-                }
-                s = (double)sf;
-            } else {
-#pragma unroll 4
-                for (; j + 1 < j1; j += 2) {
-                    r = fma(A[j * lda + i], x[j], r);
-                    r1 = fma(A[(j + 1) * lda + i], x[j + 1], r1);
-                }
-                if (j < j1) r = fma(A[j * lda + i], x[j], r);
-            }
-            r += r1;
-        }
-    } else if (dominant && diag && want_norm == 0 && HPLGB_REGEN_I2F) {
-        // the plain product with the integer t = a * 2^53 converted by the
-        // hardware (exact, |t| <= 2^52): sum t_ij x_j, then one exact scaling by
-        // 2^-53 per row; every intermediate is the a_ij version times 2^53, so
-        // the rounding is the same
-        const uint64_t step = (uint64_t)n * 0x9E3779B97F4A7C15ull;
-        uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * 0x9E3779B97F4A7C15ull;
-        double r1 = 0.0;
-        int64_t j = j0;
-        for (; j + 1 < j1; j += 2, z += 2 * step) {
-            const long long t0 = (long long)(res_mix(z) >> 11) - (1LL << 52);
-            const long long t1 = (long long)(res_mix(z + step) >> 11) - (1LL << 52);
-            r = fma(j == i ? 0.0 : (double)t0, x[j], r);
-            r1 = fma(j + 1 == i ? 0.0 : (double)t1, x[j + 1], r1);
-        }
-        if (j < j1) {
-            const long long t0 = (long long)(res_mix(z) >> 11) - (1LL << 52);
-            r = fma(j == i ? 0.0 : (double)t0, x[j], r);
-        }
-        r = (r + r1) * 0x1p-53;
-    } else if (dominant && diag && want_norm != 2) {
+    if (dominant && diag && want_norm != 2) {
         // diagonal known: plain regenerated product over the off-diagonal
         // entries, one FP64 instruction (the FMA) per entry
         const uint64_t step = (uint64_t)n * 0x9E3779B97F4A7C15ull;
@@ -192,6 +185,57 @@ __global__ void __launch_bounds__(256) k_res_partial(int64_t n, const double* __
     w.part_a[chunk * n + i] = s;
     w.part_lo[chunk * n + i] = lo;
     w.part_hi[chunk * n + i] = hi;
+}
+
+// The plain product with the regenerated dominant matrix, its diagonal left out
+// (k_res_rows and k_res_vec add diag_i x_i). Nothing is read but x, and the
+// FP64 pipe (a warp instruction in 16 clocks of the SM) bounds it, so an entry
+// costs one FP64 instruction, the FMA: a conversion of the integer entry would
+// be a second one, and the entry's bits are built by some 35 integer
+// instructions (generator included) that issue in the shadow of the FMA.
+// Every term and the order of the additions are those of the sum with the
+// entries converted from integers (two FP64 instructions an entry), so the bits
+// are too. x is staged through shared memory: read from global memory at its
+// use, its latency stood in every step (2049 rows: 26 us instead of 14).
+// n = 65536: 16.2 -> 7.7 ms with the row sums over the chunks (6.8 is the FP64
+// pipe's), 9001: 0.35 -> 0.19, 4097: 0.092 -> 0.062, 2049 and below the same. Steps of 2
+// and 8: 7.9 and 7.4 ms; 8 rounds short chunks up further.
+constexpr int kRegenStep = 4;         // entries in flight per thread
+__global__ void __launch_bounds__(256) k_res_regen(int64_t n, uint64_t key, const double* __restrict__ x, ResWs w) {
+    __shared__ double s_x[256];
+    const int64_t i0 = (int64_t)blockIdx.x * 256, i = i0 + threadIdx.x;
+    const int chunk = blockIdx.y;
+    const int64_t cw = (n + kResChunks - 1) / kResChunks;
+    const int64_t j0 = chunk * cw, j1 = std::min<int64_t>(n, j0 + cw);
+    const uint64_t gamma = 0x9E3779B97F4A7C15ull, step = (uint64_t)n * gamma;
+    uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * gamma;
+    double r[2] = {0.0, 0.0};                            // even and odd columns of the chunk
+    for (int64_t jt = j0; jt < j1; jt += 256) {
+        __syncthreads();
+        s_x[threadIdx.x] = jt + threadIdx.x < j1 ? x[jt + threadIdx.x] : 0.0;
+        __syncthreads();
+        const int cols = (int)std::min<int64_t>(256, j1 - jt);
+        const int d = (int)std::max<int64_t>(-1, std::min<int64_t>(i - jt, 512));   // the diagonal's place in the tile
+        const bool off = jt + 256 <= i0 || jt >= i0 + 256;                          // none of the block's rows has it here
+        for (int c = 0; c < cols; c += kRegenStep, z += kRegenStep * step) {        // beyond cols x is 0
+            double a[kRegenStep];
+            unsigned least = ~0u;
+#pragma unroll
+            for (int u = 0; u < kRegenStep; u++) {
+                unsigned top;
+                a[u] = gen_value_top(res_mix(z + u * step), top);
+                least = min(least, top);
+            }
+            if (least == 0)
+                for (int u = 0; u < kRegenStep; u++) a[u] = gen_value_any(res_mix(z + u * step));
+            if (!off)
+#pragma unroll
+                for (int u = 0; u < kRegenStep; u++) a[u] = c + u == d ? 0.0 : a[u];
+#pragma unroll
+            for (int u = 0; u < kRegenStep; u++) r[u & 1] = fma(a[u], s_x[c + u], r[u & 1]);
+        }
+    }
+    if (i < n) w.part_r[chunk * n + i] = r[0] + r[1];
 }
 
 __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double v) {
@@ -373,8 +417,13 @@ int launch_residual_vec(int64_t n, const double* A, int64_t lda, uint64_t key, c
     ResWs w;
     res_ws_layout(n, &w, (char*)ws);
     const double* dg = A ? nullptr : diag;
-    dim3 g1((unsigned)((n + 255) / 256), kResChunks);
-    k_res_partial<<<g1, 256, 0, s>>>(n, A, lda, key, A ? 0 : 1, dg, x, w, (sr && !anorm) ? 1 : 0);
+    const dim3 g1((unsigned)((n + 255) / 256), kResChunks);
+    const dim3 gs((unsigned)((n + kStoredRows - 1) / kStoredRows), kResChunks);
+    const bool norm = sr && !anorm;
+    if (A && norm) k_res_stored<1><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
+    else if (A) k_res_stored<0><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
+    else if (norm) k_res_partial<<<g1, 256, 0, s>>>(n, key, 1, dg, x, w, 1);
+    else k_res_regen<<<g1, 256, 0, s>>>(n, key, x, w);
     HPL_LAUNCH_CHECK();
     if (!(sr && b)) {
         k_res_vec<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, dg, x, b, w, r);
@@ -396,8 +445,10 @@ int launch_scaled_residual(int64_t n, const double* A, int64_t lda, uint64_t see
     res_ws_layout(n, &w, (char*)ws);
     HPL_CUDA_TRY(cudaMemsetAsync(w.maxima, 0, sizeof(unsigned long long) * 4, s));
     uint64_t key = res_mix(seed + 1ull * 0x9E3779B97F4A7C15ull);    // stream 0 of the generator
-    dim3 g1((unsigned)((n + 255) / 256), kResChunks);
-    k_res_partial<<<g1, 256, 0, s>>>(n, A, lda, key, kind == HPL_GEN_DIAG_DOMINANT, nullptr, x, w, 2);
+    const dim3 g1((unsigned)((n + 255) / 256), kResChunks);
+    const dim3 gs((unsigned)((n + kStoredRows - 1) / kStoredRows), kResChunks);
+    if (A) k_res_stored<2><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
+    else k_res_partial<<<g1, 256, 0, s>>>(n, key, kind == HPL_GEN_DIAG_DOMINANT, nullptr, x, w, 2);
     HPL_LAUNCH_CHECK();
     k_res_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, !A && kind == HPL_GEN_DIAG_DOMINANT, nullptr, nullptr,
                                                            x, b, w, nullptr);

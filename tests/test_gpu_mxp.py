@@ -496,3 +496,61 @@ def test_mxp_factor_same_bits_with_one_or_two_atom_stages(hpl, storage):
     finally:
         hpl.gemm_config(hpl.GEMM_PAIR_ATOMS, 2)
     assert torch.equal(F[0], F[1])
+
+
+def _seed_for_word(h, index, stream):
+    """The seed under which output `index` (from 1) of stream `stream` is the
+    word h: SplitMix64's mix is a bijection, inverted step by step."""
+    M, gamma = (1 << 64) - 1, 0x9E3779B97F4A7C15
+
+    def unshift(z, k):
+        x = z
+        for _ in range(64 // k + 1):
+            x = z ^ (x >> k)
+        return x
+
+    def unmix(z):
+        z = unshift(z, 31) * pow(0x94D049BB133111EB, -1, 1 << 64) & M
+        z = unshift(z, 27) * pow(0xBF58476D1CE4E5B9, -1, 1 << 64) & M
+        return unshift(z, 30)
+
+    return (unmix((unmix(h) - index * gamma) & M) - (stream + 1) * gamma) & M
+
+
+@pytest.mark.parametrize("t", [0, 1, -1, 2, 3 << 19, (1 << 21) - 1, -(1 << 21), 1 << 21, -(1 << 21) - 1, (1 << 52) - 1,
+                               -(1 << 52), 1 << 51, -(1 << 51)])
+def test_generated_words_near_zero(hpl, t):
+    """Entries t 2^-53 around the sizes where the upper half of |t| 2^11
+    vanishes (once in 2^31 words): the stored entry is exact, and a solve that
+    regenerates it gives the solution of the stored matrix."""
+    import torch
+    n = 5
+    for low in (0, 0x7ff):                              # bits the entry does not use
+        seed = _seed_for_word(((t + (1 << 52)) << 11) | low, 1 + 2 * n + 3, hpl.STREAM_A)
+        A = _np(hpl.generate(seed, hpl.STREAM_A, n, n))
+        assert A[3, 2] == t * 2.0 ** -53
+        A = _np(hpl.generate(seed, hpl.STREAM_A, n, n, hpl.GEN_DIAG_DOMINANT))
+        assert A[3, 2] == t * 2.0 ** -53
+        b = hpl.generate(seed, hpl.STREAM_B, n, 1)[:, 0].contiguous()
+        x, info, _ = hpl.mxp_solve(None, b, nb=8, seed=seed)
+        torch.cuda.synchronize()
+        assert info.read()["status"] == 0
+        want = np.linalg.solve(A, _np(b))
+        assert np.abs(_np(x)[:, 0] - want).max() <= 2 * 16 * n * EPS * np.linalg.cond(A, np.inf) * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 63, 255, 256, 257, 1025, 4095, 4097, 5003])
+def test_regenerated_residual_against_general(hpl, n):
+    """The refinement's residual with a regenerated matrix (chunks of n / 16
+    columns, tiles of 256, the diagonal left out and added) against the
+    acceptance check's own kernel at the same x. Either differs from the exact
+    residual by at most (n / 16 + 18) 2^-53 ||A|| ||x||; the norm is summed in
+    FP32 over the FP32 entries: n 2^-24 relative."""
+    import torch
+    seed = 21
+    b = hpl.generate(seed, hpl.STREAM_B, n, 1)[:, 0].contiguous()
+    for iters in (1, 50):
+        x, info, _ = hpl.mxp_solve(None, b, nb=256, seed=seed, refine=hpl.REFINE_IR, max_iter=iters)
+        torch.cuda.synchronize()
+        want = float(hpl.scaled_residual(None, x[:, 0].contiguous(), b, seed=seed, kind=hpl.GEN_DIAG_DOMINANT))
+        assert abs(info.read()["scaled_residual"] - want) <= 1 / 8 + 36 / n + n * 2.0 ** -24 * want
