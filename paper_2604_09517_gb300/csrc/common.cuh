@@ -146,14 +146,18 @@ __device__ __forceinline__ double gen_value_any(uint64_t h) {
         ((unsigned long long)(t < 0) << 63) | ((unsigned long long)(p - 53 + 1023) << 52) | mant;
     return __longlong_as_double((long long)bits);
 }
-// The same where top, the upper half of |t| 2^11, is not 0 (the caller looks at
-// it: 0 comes once in 2^31 words): 32-bit operations, the sign taken out with a
-// mask, one shift by the upper half's leading zeros, the leading one carried
-// into the exponent by an addition.
-__device__ __forceinline__ double gen_value_top(uint64_t h, unsigned& top) {
+// |t| 2^11 (so that the value is +-u 2^-64), m all ones where t < 0
+__device__ __forceinline__ uint64_t gen_abs(uint64_t h, unsigned& m) {
     const unsigned lo = (unsigned)h, hi = (unsigned)(h >> 32);
-    const unsigned m = ~(unsigned)((int)hi >> 31);             // all ones: t < 0
-    const uint64_t u = ((uint64_t)(hi ^ 0x80000000u ^ m) << 32 | ((lo & 0xfffff800u) ^ m)) - (uint64_t)(int64_t)(int)m;
+    m = ~(unsigned)((int)hi >> 31);
+    return ((uint64_t)(hi ^ 0x80000000u ^ m) << 32 | ((lo & 0xfffff800u) ^ m)) - (uint64_t)(int64_t)(int)m;
+}
+// The value where top, the upper half of |t| 2^11, is not 0 (the caller looks at
+// it: 0 comes once in 2^31 words): 32-bit operations, one shift by the upper
+// half's leading zeros, the leading one carried into the exponent by an addition.
+__device__ __forceinline__ double gen_value_top(uint64_t h, unsigned& top) {
+    unsigned m;
+    const uint64_t u = gen_abs(h, m);
     const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
     top = uh;
     const int s = __clz((int)uh);

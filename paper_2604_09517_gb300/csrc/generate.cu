@@ -90,31 +90,36 @@ __global__ void __launch_bounds__(256) k_dominant_diag(int64_t n, double* __rest
 // regenerate the entries). Every entry is the FP64 generated value rounded
 // once to nearest, exactly what converting a stored FP64 matrix gives.
 //
-// One pass over the entries: rows in blocks of 256 (blockIdx.x), `chunks`
-// column chunks (blockIdx.y). Per (row, chunk) the kernel writes the FP32
-// entries, the exact sum of |a_ij| / 2^-53 = |(h >> 11) - 2^52| over the
-// chunk in 128 bits (the diagonal's dominance, all j), and the FP32 sum of
-// |fl32(a_ij)| over the chunk's off-diagonal entries (||A||_inf for the
-// refinement's stopping test).
-__device__ __forceinline__ float gen_store(float* p, uint64_t h) {
-    // t = (h >> 11) - 2^52 converted by the hardware (one rounding to nearest
-    // even of the integer), then the exact scaling by 2^-53: the FP32 rounding
-    // of the FP64 value (t 2^-53) in one step
-    const long long t = (long long)(h >> 11) - (1LL << 52);
-    const float v = __ll2float_rn(t) * 0x1p-53f;
-    *p = v;
-    return v;
+// One pass over the entries: rows in blocks of 512 (blockIdx.x), two adjacent
+// rows a thread, `chunks` column chunks (blockIdx.y). Per (row, chunk) the
+// kernel writes the entries, the exact sum of |a_ij| / 2^-53 = |(h >> 11) - 2^52|
+// over the chunk in 128 bits (the diagonal's dominance, all j), and the FP32
+// sum of the stored |a_ij| over the chunk's off-diagonal entries (||A||_inf for
+// the refinement's stopping test).
+//
+// FP32: t converted by the hardware (one rounding to nearest even of the
+// integer), then the exact scaling by 2^-53; that conversion takes 16 clocks of
+// the SM a warp and bounds the kernel (n = 65536: 8.1 ms, 6.8 for the
+// conversions alone). BF16: the integer pipe bounds it (writing n = 65536 takes
+// 1.3 ms of the memory), so little is done beside the generator. The sums run
+// over u = |t| 2^11, which a mask and a subtraction take from h, in 96 bits with
+// the carry flag. The upper half of u converted toward zero to FP32's 24 bits and
+// the last of them set stands for u on the same side of every BF16 rounding
+// boundary, unless u lies on one, which needs its lower half to be 0, or the
+// upper half has fewer than 11 bits: those steps take gen_value's bits. The
+// diagonal is looked for only in the steps that meet it. n = 65536: 15.7 -> 10.0
+// ms, 16384: 1.06 -> 0.68 (two rows a thread with paired stores 10.2 ms; the
+// 64-bit conversion for every second column 10.3, for all 15.1). FP32 by fields
+// of u instead of the 64-bit conversion: 9.5 ms; in steps of 4 like BF16: 8.6.
+__device__ __forceinline__ float gen_f32(uint64_t h) {
+    return __ll2float_rn((long long)(h >> 11) - (1LL << 52)) * 0x1p-53f;
 }
-__device__ __forceinline__ float gen_store(__nv_bfloat16* p, uint64_t h) {
-    const __nv_bfloat16 v = f64_to_bf16_rn(gen_value(h));
-    *p = v;
-    return __bfloat162float(v);
-}
+
+constexpr int kGenStep = 4;           // BF16: columns in flight per thread
 
 // A32 (optional, n x n, ld n) receives the FP32 rounding of each entry as
 // well (GMRES's inner products in FP32 data).
-template <typename FT>
-__global__ void __launch_bounds__(256) k_generate_f32(uint64_t key, int64_t n, FT* __restrict__ F, int64_t ldf,
+__global__ void __launch_bounds__(256) k_generate_low(uint64_t key, int64_t n, float* __restrict__ F, int64_t ldf,
                                                       int chunks, uint64_t* __restrict__ plo,
                                                       uint64_t* __restrict__ phi, float* __restrict__ pf,
                                                       float* __restrict__ A32) {
@@ -128,14 +133,9 @@ __global__ void __launch_bounds__(256) k_generate_f32(uint64_t key, int64_t n, F
     float sf = 0.0f;
     for (int64_t j = j0; j < j1; j++, z += step) {
         const uint64_t h = sm64_mix(z);
-        const float v = gen_store(F + j * ldf + i, h);
-        if (A32) {
-            if constexpr (std::is_same<FT, float>::value) {
-                A32[j * n + i] = v;
-            } else {
-                A32[j * n + i] = __ll2float_rn((long long)(h >> 11) - (1LL << 52)) * 0x1p-53f;
-            }
-        }
+        const float v = gen_f32(h);
+        F[j * ldf + i] = v;
+        if (A32) A32[j * n + i] = v;
         const uint64_t m = h >> 11, u = m >= (1ull << 52) ? m - (1ull << 52) : (1ull << 52) - m;
         const uint64_t nl = lo + u;
         hi += (nl < lo);
@@ -145,6 +145,62 @@ __global__ void __launch_bounds__(256) k_generate_f32(uint64_t key, int64_t n, F
     plo[(int64_t)blockIdx.y * n + i] = lo;
     phi[(int64_t)blockIdx.y * n + i] = hi;
     pf[(int64_t)blockIdx.y * n + i] = sf;
+}
+
+__global__ void __launch_bounds__(256) k_generate_low(uint64_t key, int64_t n, __nv_bfloat16* __restrict__ F,
+                                                      int64_t ldf, int chunks, uint64_t* __restrict__ plo,
+                                                      uint64_t* __restrict__ phi, float* __restrict__ pf,
+                                                      float* __restrict__ A32) {
+    const int64_t i0 = (int64_t)blockIdx.x * 256, i = i0 + threadIdx.x;
+    if (i >= n) return;
+    const int64_t cw = (n + chunks - 1) / chunks;
+    const int64_t j0 = (int64_t)blockIdx.y * cw, j1 = std::min<int64_t>(n, j0 + cw);
+    const uint64_t step = (uint64_t)n * kGamma;
+    uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * kGamma;
+    unsigned s0 = 0, s1 = 0, s2 = 0;                     // sum of u, 96 bits
+    float sf = 0.0f;
+    __nv_bfloat16* f = F + j0 * ldf + i;
+    float* f32 = A32 ? A32 + j0 * n + i : nullptr;
+    auto columns = [&](int64_t j, auto count, bool diag) {
+        constexpr int N = decltype(count)::value;
+        float v[N];
+        unsigned top = ~0u, low = ~0u;
+#pragma unroll
+        for (int c = 0; c < N; c++) {
+            const uint64_t h = sm64_mix(z + c * step);
+            unsigned m;
+            const uint64_t u = gen_abs(h, m);
+            const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
+            asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+                : "+r"(s0), "+r"(s1), "+r"(s2) : "r"(ul), "r"(uh));
+            top = min(top, uh);
+            low = min(low, ul);
+            v[c] = __uint_as_float(__float_as_uint(__uint2float_rz(uh)) | 1u | (m & 0x80000000u)) * 0x1p-32f;
+            if (f32) f32[c * n] = gen_f32(h);
+        }
+        const bool again = low == 0 || top < 1024u;
+#pragma unroll
+        for (int c = 0; c < N; c++) {
+            __nv_bfloat16 b = __float2bfloat16_rn(v[c]);
+            if (again) b = f64_to_bf16_rn(gen_value(sm64_mix(z + c * step)));
+            f[c * ldf] = b;
+            sf += diag && j + c == i ? 0.0f : fabsf(__bfloat162float(b));
+        }
+        z += N * step;
+        f += N * ldf;
+        if (f32) f32 += N * n;
+    };
+    int64_t j = j0;
+    for (; j + kGenStep <= j1; j += kGenStep) {
+        if (j + kGenStep <= i0 || j >= i0 + 256) columns(j, std::integral_constant<int, kGenStep>(), false);
+        else columns(j, std::integral_constant<int, kGenStep>(), true);
+    }
+    for (; j < j1; j++) columns(j, std::integral_constant<int, 1>(), true);
+    const int64_t o = (int64_t)blockIdx.y * n + i;
+    const uint64_t lo = (uint64_t)s1 << 32 | s0;             // the sum of |t| is the sum of u over 2^11
+    plo[o] = lo >> 11 | (uint64_t)s2 << 53;
+    phi[o] = s2 >> 11;
+    pf[o] = sf;
 }
 
 // Per row: the exact row sum over the chunks, rounded once, is the FP64
@@ -185,12 +241,12 @@ int launch_generate_dominant_f32(uint64_t seed, int64_t n, void* F, int64_t ldf,
     const dim3 g1((unsigned)((n + 255) / 256), (unsigned)chunks), g2((unsigned)((n + 255) / 256));
     if (bf16) {
         __nv_bfloat16* Fb = (__nv_bfloat16*)F;
-        k_generate_f32<<<g1, 256, 0, s>>>(key, n, Fb, ldf, chunks, plo, phi, pf, A32);
+        k_generate_low<<<g1, 256, 0, s>>>(key, n, Fb, ldf, chunks, plo, phi, pf, A32);
         HPL_LAUNCH_CHECK();
         k_dominant_diag_fin<<<g2, 256, 0, s>>>(n, chunks, plo, phi, diag, Fb, ldf, pf, A32);
     } else {
         float* Ff = (float*)F;
-        k_generate_f32<<<g1, 256, 0, s>>>(key, n, Ff, ldf, chunks, plo, phi, pf, A32);
+        k_generate_low<<<g1, 256, 0, s>>>(key, n, Ff, ldf, chunks, plo, phi, pf, A32);
         HPL_LAUNCH_CHECK();
         k_dominant_diag_fin<<<g2, 256, 0, s>>>(n, chunks, plo, phi, diag, Ff, ldf, pf, A32);
     }

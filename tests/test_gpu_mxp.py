@@ -554,3 +554,26 @@ def test_regenerated_residual_against_general(hpl, n):
         torch.cuda.synchronize()
         want = float(hpl.scaled_residual(None, x[:, 0].contiguous(), b, seed=seed, kind=hpl.GEN_DIAG_DOMINANT))
         assert abs(info.read()["scaled_residual"] - want) <= 1 / 8 + 36 / n + n * 2.0 ** -24 * want
+
+
+@pytest.mark.parametrize("t", [
+    0x101 << 30, 0x103 << 30, (0x101 << 30) + 1, (0x103 << 30) - 1, -(0x101 << 30), -(0x103 << 30) - 1,     # BF16 ties
+    (0x101 << 43), (0x1ff << 43) + (1 << 42), (0x1ff << 42), -(0x1ff << 43),
+    0x101 << 20, (0x101 << 20) + 1, 0x1ff << 22, 0x101, -0x103, 0xff, 3, 0, -1, -(1 << 52), (1 << 52) - 1,
+    (1 << 31) - 1, (1 << 31) + (1 << 23), (1 << 30) + (1 << 22), (0x1000001 << 20), (0x1000003 << 20) + 1,      # FP32 ties
+])
+def test_generated_words_rounded_once(hpl, orc, t):
+    """Regenerated entries on and beside the rounding boundaries of BF16 and
+    FP32, and where few leading bits are left: the working copy holds the one
+    rounding of t 2^-53."""
+    import torch
+    n = 5
+    seed = _seed_for_word(((t + (1 << 52)) << 11) | 0x2a5, 1 + 2 * n + 3, hpl.STREAM_A)
+    b = hpl.generate(seed, hpl.STREAM_B, n, 1)[:, 0].contiguous()
+    for storage in (hpl.STORAGE_FP32, hpl.STORAGE_BF16):
+        _, info, ws = hpl.mxp_solve(None, b, nb=8, seed=seed, storage=storage)
+        torch.cuda.synchronize()
+        assert info.read()["status"] == 0
+        F, _ = hpl.mxp_factor_views(ws, n, 8, storage=storage)
+        v = t * 2.0 ** -53
+        assert float(F[3, 2]) == (orc.round_bf16_d(v) if storage == hpl.STORAGE_BF16 else float(np.float32(v)))
