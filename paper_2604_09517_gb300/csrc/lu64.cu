@@ -855,6 +855,62 @@ __global__ void __launch_bounds__(256) k_trsm_lunit(double* __restrict__ A, int6
         for (int i = g; i < kk; i += 16) A[col * lda + r0 + i] = xs[i * kTrsmCols + c];
 }
 
+// The same for 64 < kk <= 256 and few columns in one launch (blocked by 64, the
+// solves and the products between them are seven launches of 10 to 18 us each in
+// series): thread r keeps row r of x for NC columns in registers, warp b solves
+// rows 32 b .. 32 b + 31 by shuffles and publishes them, and the warps below
+// subtract their part. The rows of L need no staging (each thread reads its own,
+// 32 entries ahead of their use). What bounds it: the chain of kk steps, a
+// shuffle and an FMA each, and the FMAs of NC columns on one SM. kk = 256 and 256
+// columns: 115 -> 50 us; kk = 128 and 128 columns: 45 -> 14 us. n = 3001 23.6 ->
+// 22.5 ms, n = 8192 with the emulated update 68.3 -> 65.5, n = 12000 148 -> 145.
+// One launch for many columns as well (4 per CTA) loses: 2489 columns 320 -> 499
+// us, because the chain is walked once per wave of CTAs.
+constexpr int kTrsmRows = 256;
+template <int NC>
+__global__ void __launch_bounds__(kTrsmRows) k_trsm_lunit_rows(double* __restrict__ A, int64_t lda, int64_t r0, int kk,
+                                                               int64_t cb, int64_t ce) {
+    __shared__ __align__(16) double xs[2][32][NC];           // the published rows, alternating
+    const int r = threadIdx.x, lane = r & 31, warp = r >> 5, nblk = blockDim.x >> 5;
+    const int64_t col0 = cb + (int64_t)blockIdx.x * NC;
+    const double* L = A + r0 * lda + r0 + r;                 // L(r, j) = L[j * lda]
+    const bool row = r < kk;
+    double x[NC], ld[32], lu[32];
+#pragma unroll
+    for (int c = 0; c < NC; c++) x[c] = row && col0 + c < ce ? A[(col0 + c) * lda + r0 + r] : 0.0;
+#pragma unroll
+    for (int j = 0; j < 32; j++) {
+        ld[j] = row && j < lane ? L[(int64_t)(32 * warp + j) * lda] : 0.0;
+        lu[j] = row && warp > 0 ? L[(int64_t)j * lda] : 0.0;
+    }
+    for (int b = 0; b < nblk; b++) {
+        if (warp == b) {
+#pragma unroll
+            for (int j = 0; j < 31; j++)
+#pragma unroll
+                for (int c = 0; c < NC; c++) {
+                    const double xj = __shfl_sync(0xffffffffu, x[c], j);
+                    if (lane > j) x[c] = fma(-ld[j], xj, x[c]);
+                }
+#pragma unroll
+            for (int c = 0; c < NC; c++) xs[b & 1][lane][c] = x[c];
+        }
+        __syncthreads();
+        if (warp > b) {
+#pragma unroll
+            for (int j = 0; j < 32; j++)
+#pragma unroll
+                for (int c = 0; c < NC; c++) x[c] = fma(-lu[j], xs[b & 1][j][c], x[c]);
+            if (row && warp > b + 1)
+#pragma unroll
+                for (int j = 0; j < 32; j++) lu[j] = L[(int64_t)(32 * (b + 1) + j) * lda];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; c++)
+        if (row && col0 + c < ce) A[(col0 + c) * lda + r0 + r] = x[c];
+}
+
 // ---------------------------------------------------------------------------
 // DGEMM: C -= A * B in FP64 with DFMA. TB x TB CTA tile (64, or 32 when
 // 64-wide tiles would leave SMs idle: one 64 x 64 x 64 tile is ~60 us of a
@@ -1175,14 +1231,29 @@ static int launch_trsm(double* A, int64_t lda, int64_t r0, int kk, int64_t cb, i
         return HPL_OK;
     }
     if (g_trsm_blocked) {
-        // Blocked by 64: each diagonal block solved by the shared-memory TRSM,
-        // the rows below it updated by the DFMA product. Every x_i still
-        // receives fma(-L_ij, x_j, x_i) for j = 0, 1, ... in order (both
-        // kernels accumulate in place, in k order), so the result is
-        // bit-identical to the one-kernel TRSM; three quarters of the flops
-        // (kk = 256) run on the update kernel's tiles.
-        for (int b0 = 0; b0 < kk; b0 += 64) {
-            const int bk = std::min(64, kk - b0);
+        // Few columns (one or two per SM; n = 3001, look-ahead and panel columns:
+        // 22.5 ms, with the line at one per SM 23.0, at four 22.5): up to kTrsmRows
+        // rows in one launch. Otherwise blocked by 64: each diagonal block solved by the
+        // shared-memory TRSM. The rows below a block are updated by the DFMA
+        // product. Every x_i receives fma(-L_ij, x_j, x_i) for j = 0, 1, ... in
+        // order whichever way (all these kernels accumulate in place, in k
+        // order), so the result is bit-identical to the one-kernel TRSM; blocked
+        // by 64, three quarters of the flops (kk = 256) run on the update
+        // kernel's tiles.
+        const int64_t nx = ce - cb;
+        const bool few = nx <= 2 * kNumSMsGB300;
+        if (few && kk <= kTrsmRows) {
+            const unsigned threads = (unsigned)((kk + 31) / 32 * 32);
+            if (nx <= kNumSMsGB300)
+                k_trsm_lunit_rows<1><<<(unsigned)nx, threads, 0, s>>>(A, lda, r0, kk, cb, ce);
+            else
+                k_trsm_lunit_rows<2><<<(unsigned)((nx + 1) / 2), threads, 0, s>>>(A, lda, r0, kk, cb, ce);
+            HPL_LAUNCH_CHECK();
+            return HPL_OK;
+        }
+        const int step = few ? kTrsmRows : 64;
+        for (int b0 = 0; b0 < kk; b0 += step) {
+            const int bk = std::min(step, kk - b0);
             int st = launch_trsm(A, lda, r0 + b0, bk, cb, ce, s);
             if (st) return st;
             if (b0 + bk < kk) {

@@ -587,3 +587,27 @@ def test_warp_trsm_bits(hpl, n, nb):
         hpl.lu_config(hpl.LU_TRSM_BLOCKED, 1)
     for A, ipiv in outs[1:]:
         assert torch.equal(A, outs[0][0]) and torch.equal(ipiv, outs[0][1])
+
+
+@pytest.mark.parametrize("n,nb", [(90, 65), (257, 256), (408, 256), (409, 256), (560, 256), (561, 256), (330, 97),
+                                  (640, 129), (700, 300), (1100, 512)])
+def test_one_launch_trsm_bits(hpl, n, nb):
+    """The one-launch TRSM of few columns (blocks of 65 to 256 rows, ragged
+    last warps, one column to two per SM, both sides of that line, blocks above
+    256 rows in pieces) gives the bits of the one-kernel TRSM."""
+    import torch
+    A0 = hpl.generate(17, hpl.STREAM_A, n, n)
+    outs = []
+    try:
+        for blocked, la in ((0, 0), (1, 0), (1, 1)):
+            hpl.lu_config(hpl.LU_TRSM_BLOCKED, blocked)
+            A = hpl.colmajor(n, n)
+            A.copy_(A0)
+            ipiv, info = hpl.lu_factor(A, nb=nb, lookahead=la)
+            torch.cuda.synchronize()
+            assert info.read()["status"] == 0
+            outs.append((A, ipiv))
+    finally:
+        hpl.lu_config(hpl.LU_TRSM_BLOCKED, 1)
+    for A, ipiv in outs[1:]:
+        assert torch.equal(A, outs[0][0]) and torch.equal(ipiv, outs[0][1])
