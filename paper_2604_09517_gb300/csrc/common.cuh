@@ -115,22 +115,6 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
     return r;
 }
-__device__ __forceinline__ double ld_cluster_f64(uint32_t caddr) {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(caddr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_cluster_f64(uint32_t caddr, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(caddr), "d"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_s64(uint32_t caddr, long long v) {
-    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(caddr), "l"(v) : "memory");
-}
-__device__ __forceinline__ long long ld_cluster_s64(uint32_t caddr) {
-    long long v;
-    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(caddr) : "memory");
-    return v;
-}
 
 // The generator's entry value (h >> 11) * 2^-53 - 0.5 from a SplitMix64
 // output h, built with integer operations only: FP64 conversions and

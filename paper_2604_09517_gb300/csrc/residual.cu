@@ -73,27 +73,26 @@ __device__ __forceinline__ float abs_as_float(double a) {
     return __int_as_float((e << 23) | (int)((u >> 29) & 0x7fffff));
 }
 
-// A stored. NORM: 0 skips the row sums of |a_ij| (plain matrix-vector product),
-// 1 sums them in FP32 from abs_as_float (the refinement's stopping test),
-// 2 sums them in FP64 (the HPL acceptance check). The product alone is within
-// 10 % of the FP64 pipe's time (n = 16384: 471 us, 426 at two FMA a clock and SM;
-// 321 for reading A). A warp per block: all blocks are resident at once up to
+// A stored. NORM sums |a_ij| along the rows as well, in FP64 (the HPL acceptance
+// check); without it this is the plain matrix-vector product of the refinement.
+// The product alone is within 10 % of the FP64 pipe's time (n = 16384: 471 us,
+// 426 at two FMA a clock and SM; 321 for reading A). A warp per block: all blocks are resident at once up to
 // n = 9700 and the SMs' shares differ least (32 / 64 / 256 rows per block: n =
 // 4096 43 / 54 / 60 us, 8192 125 / 126 / 144, 16384 471 / 477 / 514, 49152 4025 /
 // 4055 / 4153); four pairs of columns in flight (two: 16384 567 us; eight gain 1 to
 // 5 % above 20000 rows and lose up to 8 % below).
 constexpr int kStoredRows = 32;
 constexpr int kStoredUnroll = 4;      // pairs of columns in flight
-template <int NORM>
-__global__ void __launch_bounds__(kStoredRows) k_res_stored(int64_t n, const double* __restrict__ A, int64_t lda,
-                                                    const double* __restrict__ x, ResWs w) {
+template <bool NORM>
+__global__ void __launch_bounds__(kStoredRows) k_res_stored(int64_t n, const double* __restrict__ A,
+                                                            int64_t lda, const double* __restrict__ x, ResWs w) {
     const int64_t i = (int64_t)blockIdx.x * kStoredRows + threadIdx.x;
     const int chunk = blockIdx.y;
     const int64_t cw = (n + kResChunks - 1) / kResChunks;
     const int64_t j0 = chunk * cw, j1 = std::min<int64_t>(n, j0 + cw);
     if (i >= n) return;
     double r = 0.0, s = 0.0;
-    if (NORM == 2) {
+    if (NORM) {
 #pragma unroll 8
         for (int64_t j = j0; j < j1; j++) {
             double a = A[j * lda + i];
@@ -103,21 +102,14 @@ __global__ void __launch_bounds__(kStoredRows) k_res_stored(int64_t n, const dou
     } else {
         // two interleaved FP64 accumulators shorten the dependent FMA chain
         double r1 = 0.0;
-        float sf = 0.0f;
         int64_t j = j0;
 #pragma unroll kStoredUnroll
         for (; j + 1 < j1; j += 2) {
             double a0 = A[j * lda + i], a1 = A[(j + 1) * lda + i];
             r = fma(a0, x[j], r);
             r1 = fma(a1, x[j + 1], r1);
-            if (NORM) sf += abs_as_float(a0) + abs_as_float(a1);
         }
-        if (j < j1) {
-            double a0 = A[j * lda + i];
-            r = fma(a0, x[j], r);
-            if (NORM) sf += abs_as_float(a0);
-        }
-        s = (double)sf;
+        if (j < j1) r = fma(A[j * lda + i], x[j], r);
         r += r1;
     }
     w.part_r[chunk * n + i] = r;
@@ -128,13 +120,11 @@ __global__ void __launch_bounds__(kStoredRows) k_res_stored(int64_t n, const dou
     }
 }
 
-// The entries regenerated from key (hpl_generate's definition), with their row
-// sums (want_norm as NORM above, 1 or 2); for the dominant matrix the diagonal
-// is skipped here and added per row later, either from the exact row sums
-// accumulated here (diag == NULL) or from diag.
+// The entries regenerated from key (hpl_generate's definition), with their FP64
+// row sums; for the dominant matrix the diagonal is skipped here and added per
+// row later from the exact row sums accumulated here.
 __global__ void __launch_bounds__(256) k_res_partial(int64_t n, uint64_t key, int dominant,
-                                                     const double* __restrict__ diag, const double* __restrict__ x,
-                                                     ResWs w, int want_norm) {
+                                                     const double* __restrict__ x, ResWs w) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int chunk = blockIdx.y;
     const int64_t cw = (n + kResChunks - 1) / kResChunks;
@@ -142,44 +132,20 @@ __global__ void __launch_bounds__(256) k_res_partial(int64_t n, uint64_t key, in
     if (i >= n) return;
     double r = 0.0, s = 0.0;
     uint64_t lo = 0, hi = 0;
-    if (dominant && diag && want_norm != 2) {
-        // diagonal known: plain regenerated product over the off-diagonal
-        // entries, one FP64 instruction (the FMA) per entry
-        const uint64_t step = (uint64_t)n * 0x9E3779B97F4A7C15ull;
-        uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * 0x9E3779B97F4A7C15ull;
-        double r1 = 0.0;
-        float sf = 0.0f;
-        int64_t j = j0;
-        for (; j + 1 < j1; j += 2, z += 2 * step) {
-            const double a0 = j == i ? 0.0 : gen_value(res_mix(z));
-            const double a1 = j + 1 == i ? 0.0 : gen_value(res_mix(z + step));
-            r = fma(a0, x[j], r);
-            r1 = fma(a1, x[j + 1], r1);
-            if (want_norm == 1) sf += abs_as_float(a0) + abs_as_float(a1);
+    const uint64_t step = (uint64_t)n * 0x9E3779B97F4A7C15ull;
+    uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * 0x9E3779B97F4A7C15ull;
+    for (int64_t j = j0; j < j1; j++, z += step) {
+        uint64_t h = res_mix(z);
+        double a = gen_value(h);
+        if (dominant) {
+            uint64_t m = h >> 11, u = m >= (1ull << 52) ? m - (1ull << 52) : (1ull << 52) - m;
+            uint64_t nl = lo + u;
+            hi += (nl < lo);
+            lo = nl;
+            if (j == i) continue;     // the diagonal is added once the row sum is known
         }
-        if (j < j1) {
-            const double a0 = j == i ? 0.0 : gen_value(res_mix(z));
-            r = fma(a0, x[j], r);
-            if (want_norm == 1) sf += abs_as_float(a0);
-        }
-        r += r1;
-        if (want_norm == 1) s = (double)sf;
-    } else {
-        const uint64_t step = (uint64_t)n * 0x9E3779B97F4A7C15ull;
-        uint64_t z = key + ((uint64_t)j0 * (uint64_t)n + (uint64_t)i + 1) * 0x9E3779B97F4A7C15ull;
-        for (int64_t j = j0; j < j1; j++, z += step) {
-            uint64_t h = res_mix(z);
-            double a = gen_value(h);
-            if (dominant) {
-                uint64_t m = h >> 11, u = m >= (1ull << 52) ? m - (1ull << 52) : (1ull << 52) - m;
-                uint64_t nl = lo + u;
-                hi += (nl < lo);
-                lo = nl;
-                if (j == i) continue;     // the diagonal is added once the row sum is known
-            }
-            r = fma(a, x[j], r);
-            s += fabs(a);
-        }
+        r = fma(a, x[j], r);
+        s += fabs(a);
     }
     w.part_r[chunk * n + i] = r;
     w.part_a[chunk * n + i] = s;
@@ -409,20 +375,17 @@ size_t residual_ws_bytes(int64_t n) { return res_ws_layout(n > 0 ? n : 1, nullpt
 // or, with A == NULL, the dominant generated matrix of key (the generator's
 // stream key) regenerated entry by entry with its diagonal taken from diag.
 // With sr != NULL (and b != NULL) also the scaled residual of x, with
-// ||A||_inf read from anorm (device) if given, else summed here in FP32.
+// ||A||_inf read from anorm (device).
 int launch_residual_vec(int64_t n, const double* A, int64_t lda, uint64_t key, const double* diag,
                         const double* anorm, const double* x, const double* b, double* r, double* sr, void* ws,
                         cudaStream_t s) {
-    if (!A && !diag) return HPL_ERR_INVALID;
+    if ((!A && !diag) || (sr && !anorm)) return HPL_ERR_INVALID;
     ResWs w;
     res_ws_layout(n, &w, (char*)ws);
     const double* dg = A ? nullptr : diag;
     const dim3 g1((unsigned)((n + 255) / 256), kResChunks);
     const dim3 gs((unsigned)((n + kStoredRows - 1) / kStoredRows), kResChunks);
-    const bool norm = sr && !anorm;
-    if (A && norm) k_res_stored<1><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
-    else if (A) k_res_stored<0><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
-    else if (norm) k_res_partial<<<g1, 256, 0, s>>>(n, key, 1, dg, x, w, 1);
+    if (A) k_res_stored<false><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
     else k_res_regen<<<g1, 256, 0, s>>>(n, key, x, w);
     HPL_LAUNCH_CHECK();
     if (!(sr && b)) {
@@ -447,8 +410,8 @@ int launch_scaled_residual(int64_t n, const double* A, int64_t lda, uint64_t see
     uint64_t key = res_mix(seed + 1ull * 0x9E3779B97F4A7C15ull);    // stream 0 of the generator
     const dim3 g1((unsigned)((n + 255) / 256), kResChunks);
     const dim3 gs((unsigned)((n + kStoredRows - 1) / kStoredRows), kResChunks);
-    if (A) k_res_stored<2><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
-    else k_res_partial<<<g1, 256, 0, s>>>(n, key, kind == HPL_GEN_DIAG_DOMINANT, nullptr, x, w, 2);
+    if (A) k_res_stored<true><<<gs, kStoredRows, 0, s>>>(n, A, lda, x, w);
+    else k_res_partial<<<g1, 256, 0, s>>>(n, key, kind == HPL_GEN_DIAG_DOMINANT, x, w);
     HPL_LAUNCH_CHECK();
     k_res_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, !A && kind == HPL_GEN_DIAG_DOMINANT, nullptr, nullptr,
                                                            x, b, w, nullptr);
