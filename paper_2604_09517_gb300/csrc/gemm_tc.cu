@@ -129,6 +129,7 @@ struct Params {
     int group_m;           // row tiles per band of the tile walk
     uint16_t* C16;         // optional BF16 copy of a stored product (sub = 0), row-major, ld16 a multiple of 8
     long long ld16;
+    int groups, kstep;     // grouped launch: products 0 .. groups - 1, see k_gemm_tc
 };
 
 
@@ -266,7 +267,15 @@ __device__ __forceinline__ void tile_coords(int t, int mt_count, int nt_count, i
 
 // C is FP32, or BF16 for a working matrix stored in BF16 (ld_f / st_f: read
 // widened to FP32, the FP32 result rounded to nearest even when stored).
-template <int KIND, int BN, typename CT, bool TMA_EPI>
+//
+// GROUPS: several products of the same operands in one launch, for the sliced
+// FP64 update of few columns: product g contracts the first (g + 1) kstep of A's
+// K with the last (g + 1) kstep of B's and goes to C's columns from g N on. The
+// longest products' tiles come first. m = 7936, 256 columns, kb = 256: 76 us
+// against eleven launches of one wave each (6 to 17 us and the gaps between
+// them, 155 us); LU with the sliced update at n = 8192 65.5 -> 62.1 ms, n = 12000
+// 144.7 -> 139.5.
+template <int KIND, int BN, typename CT, bool TMA_EPI, bool GROUPS = false>
 __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               const __grid_constant__ CUtensorMap tmC, Params p) {
@@ -280,8 +289,14 @@ __global__ void __launch_bounds__(THREADS, 1)
     unsigned char* tiles = (unsigned char*)(((uintptr_t)dsm + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mt_count = (p.M + BM - 1) / BM, nt_count = (p.N + BN - 1) / BN;
-    const int ntiles = mt_count * nt_count;
-    const int nk = (p.K + BK - 1) / BK;
+    const int per_group = mt_count * nt_count;
+    const int ntiles = GROUPS ? p.groups * per_group : per_group;
+    // tile t's product, K steps and coordinates
+    auto tile = [&](int t, int& mt, int& nt, int& g, int& nk) {
+        g = GROUPS ? p.groups - 1 - t / per_group : 0;
+        nk = GROUPS ? (g + 1) * (p.kstep / BK) : (p.K + BK - 1) / BK;
+        tile_coords(GROUPS ? t % per_group : t, mt_count, nt_count, p.group_m, mt, nt);
+    };
     const uint64_t deadline = globaltimer_ns() + (uint64_t)p.timeout_ns;
 
     if (threadIdx.x == 0) {
@@ -316,8 +331,9 @@ __global__ void __launch_bounds__(THREADS, 1)
             uint32_t it = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                int mt, nt;
-                tile_coords(t, mt_count, nt_count, p.group_m, mt, nt);
+                int mt, nt, g, nk;
+                tile(t, mt, nt, g, nk);
+                const int bk0 = GROUPS ? (p.groups - 1 - g) * p.kstep : 0;
                 for (int kb = 0; kb < nk; kb++, it++) {
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1;
@@ -325,7 +341,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     unsigned char* sa = tiles + s * STAGE_BYTES;
                     mbar_expect_tx(&full_bar[s], STAGE_BYTES);
                     tma_load_2d(sa, &tmA, &full_bar[s], kb * BK, mt * BM);
-                    tma_load_2d(sa + A_BYTES, &tmB, &full_bar[s], kb * BK, nt * BN);
+                    tma_load_2d(sa + A_BYTES, &tmB, &full_bar[s], bk0 + kb * BK, nt * BN);
                 }
             }
             if (!ok) {
@@ -345,6 +361,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (!mbar_wait(&tempty_bar[acc], aph ^ 1, deadline, &s_abort, p.err)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
+                int mt, nt, g, nk;
+                tile(t, mt, nt, g, nk);
                 for (int kb = 0; kb < nk; kb++, it++) {
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1;
@@ -374,8 +392,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         float* stage = (float*)(tiles + STAGES * STAGE_BYTES) + (warp - 2) * EPI_CHUNK_FLOATS;
         uint32_t tcount = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, tcount++) {
-            int mt, nt;
-            tile_coords(t, mt_count, nt_count, p.group_m, mt, nt);
+            int mt, nt, g, nk;
+            tile(t, mt, nt, g, nk);
             const uint32_t acc = tcount & 1, aph = (tcount >> 1) & 1;
             const int row0 = mt * BM + quarter * 32;
             const int row = row0 + lane;
@@ -396,7 +414,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
                 if (c * 32 < ncol)
                     epi_chunk_tma(&tmC, stage, r, rs, p.sb, cbase + c * 32, ncol - c * 32, p.sub, row0,
-                                  cbase + c * 32, lane, p.C16, p.ld16, p.M);
+                                  g * p.N + cbase + c * 32, lane, p.C16, p.ld16, p.M);
             }
         }
         if (lane == 0) bulk_wait_all();
@@ -414,13 +432,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         constexpr int CHUNKS = BN / 2 / 32;
         uint32_t tcount = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, tcount++) {
-            int mt, nt;
-            tile_coords(t, mt_count, nt_count, p.group_m, mt, nt);
+            int mt, nt, g, nk;
+            tile(t, mt, nt, g, nk);
             const uint32_t acc = tcount & 1, aph = (tcount >> 1) & 1;
             const int row = mt * BM + row_in_tile;
             const bool row_ok = row < p.M;
             const int cbase = nt * BN + half * (BN / 2);
-            CT* cp = (CT*)p.C + (long long)cbase * p.ldc + row;
+            CT* cp = (CT*)p.C + ((long long)g * p.N + cbase) * p.ldc + row;
             const int ncol = min(BN / 2, p.N - cbase);      // valid columns of this half (may be <= 0)
             float cv[32];
             if (p.sub) {
@@ -862,18 +880,18 @@ static bool tma_epilogue_ok(const CT* C, int64_t ldc) {
     }
 }
 
-template <int KIND, int BN, typename CT, bool TMA_EPI>
+template <int KIND, int BN, typename CT, bool TMA_EPI, bool GROUPS = false>
 static int launch_kind_epi(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const Params& p,
                            int grid, cudaStream_t s) {
     static std::atomic<bool> attr_set[kMaxDevices];
     const int dv = device_slot();
     if (dv < 0) return HPL_ERR_CUDA;
     if (!attr_set[dv].load()) {
-        HPL_CUDA_TRY(cudaFuncSetAttribute((const void*)k_gemm_tc<KIND, BN, CT, TMA_EPI>,
+        HPL_CUDA_TRY(cudaFuncSetAttribute((const void*)k_gemm_tc<KIND, BN, CT, TMA_EPI, GROUPS>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_smem<BN, TMA_EPI>()));
         attr_set[dv].store(true);
     }
-    k_gemm_tc<KIND, BN, CT, TMA_EPI><<<grid, THREADS, dyn_smem<BN, TMA_EPI>(), s>>>(ma, mb, mc, p);
+    k_gemm_tc<KIND, BN, CT, TMA_EPI, GROUPS><<<grid, THREADS, dyn_smem<BN, TMA_EPI>(), s>>>(ma, mb, mc, p);
     HPL_LAUNCH_CHECK();
     return HPL_OK;
 }
@@ -917,6 +935,8 @@ static int launch_kind(int64_t M, int64_t N, int64_t K, const void* A, int64_t l
     p.sb = sb;
     p.C16 = C16;
     p.ld16 = ld16;
+    p.groups = 1;
+    p.kstep = 0;
     p.group_m = g_group_m_override > 0 ? g_group_m_override : group_m<KIND>();
     if (tma_epi) return launch_kind_epi<KIND, BN, CT, true>(ma, mb, mc, p, grid, s);
     return launch_kind_epi<KIND, BN, CT, false>(ma, mb, mc, p, grid, s);
@@ -993,6 +1013,8 @@ static int launch_pair(int64_t M, int64_t N, int64_t K, const void* A, int64_t l
     p.sb = sb;
     p.C16 = C16;
     p.ld16 = ld16;
+    p.groups = 1;
+    p.kstep = 0;
     p.group_m = g_group_m_override > 0 ? g_group_m_override : GROUP_M_PAIR;
     if (two_atoms) {
         if (tma_epi)
@@ -1038,6 +1060,48 @@ int launch_gemm_bf16(int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t
                                        max_ctas, s);
     return tc::launch_kind<0, 256>(M, N, K, A, lda, B, ldb, nullptr, nullptr, C, ldc, sub, err, timeout_ns, max_ctas,
                                    s);
+}
+
+// The products g = 0 .. groups - 1 of the same operands (K contiguous, groups
+// kstep of it): C_g (M x N, ld M, at C + g M N) = A(:, first (g + 1) kstep)
+// B(:, last (g + 1) kstep)^T, in one launch of the single-CTA kernel on 128 x 128
+// tiles. Returns 1 where the form does not hold: K steps that straddle a stage,
+// product columns that end inside a 32-column chunk of the epilogue, or products
+// that fill the SM pairs by themselves (the pair kernel, one launch each, is
+// faster then).
+int launch_gemm_bf16_groups(int64_t M, int64_t N, int64_t kstep, int groups, const uint16_t* A, int64_t lda,
+                            const uint16_t* B, int64_t ldb, float* C, int* err, int64_t timeout_ns, cudaStream_t s) {
+    constexpr int BN = 128, BK = tc::BKB / 2;
+    const int64_t K = groups * kstep;
+    if (M <= 0 || N <= 0 || kstep <= 0 || kstep % BK || N % 32) return 1;
+    if (tc::pair_tiles(M, N, tc::tma_epilogue_ok(C, M)) || !tc::narrow_tiles(M, N)) return 1;
+    const int64_t tiles = ((M + tc::BM - 1) / tc::BM) * ((N + BN - 1) / BN) * groups;
+    if (K > 0x7fffffff || N * groups > 0x7fffffff || tiles > 0x7fffffff) return 1;
+    if (lda < K || ldb < K || lda % 8 || ldb % 8 || (((uintptr_t)A | (uintptr_t)B) & 15)) return 1;
+    CUtensorMap ma, mb, mc;
+    int st = tc::make_map(&ma, A, M, K, lda, tc::BM, 2);
+    if (st) return st;
+    if ((st = tc::make_map(&mb, B, N, K, ldb, BN, 2))) return st;
+    const bool tma_epi = tc::tma_epilogue_ok(C, M);
+    memset(&mc, 0, sizeof(mc));
+    if (tma_epi && (st = tc::make_map_c(&mc, C, M, N * groups, M))) return st;
+    int dev = 0, sms = kNumSMsGB300;
+    HPL_CUDA_TRY(cudaGetDevice(&dev));
+    HPL_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    tc::Params p = {};
+    p.M = (int)M;
+    p.N = (int)N;
+    p.K = (int)K;
+    p.C = C;
+    p.ldc = M;
+    p.err = err;
+    p.timeout_ns = timeout_ns > 0 ? timeout_ns : kDefaultTimeoutNs;
+    p.group_m = tc::group_m<0>();
+    p.groups = groups;
+    p.kstep = (int)kstep;
+    const int grid = (int)std::min<int64_t>(tiles, sms);
+    if (tma_epi) return tc::launch_kind_epi<0, BN, float, true, true>(ma, mb, mc, p, grid, s);
+    return tc::launch_kind_epi<0, BN, float, false, true>(ma, mb, mc, p, grid, s);
 }
 
 // A stored BF16 product C = A B^T (FP32 C) that also writes C rounded to BF16,

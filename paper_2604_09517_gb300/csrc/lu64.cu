@@ -1146,6 +1146,8 @@ __global__ void __launch_bounds__(256) k_emu_combine(int64_t m, int64_t nc, cons
 
 int launch_gemm_bf16(int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb,
                      float* C, int64_t ldc, int sub, int* err, int64_t timeout_ns, int max_ctas, cudaStream_t s);
+int launch_gemm_bf16_groups(int64_t M, int64_t N, int64_t kstep, int groups, const uint16_t* A, int64_t lda,
+                            const uint16_t* B, int64_t ldb, float* C, int* err, int64_t timeout_ns, cudaStream_t s);
 
 // Slices of one step: L21 (m x kb, ld ldl; none when m is 0) and the columns
 // col0 .. col0+nn of the block row U12 (U: kb x nn, ld ldu).
@@ -1174,12 +1176,15 @@ static int emu_update(const LuWs& w, int64_t m, int64_t nn, int kb, int64_t col0
     const int64_t lds = (int64_t)kEmuSlices * kbp;
     for (int64_t j0 = 0; j0 < nn; j0 += kEmuChunk) {
         const int64_t nc = std::min<int64_t>(kEmuChunk, nn - j0);
-        for (int g = 2; g <= kEmuSlices + 1; g++) {
+        int st = launch_gemm_bf16_groups(m, nc, kbp, kEmuSlices, w.sA, lds, w.sB + (col0 + j0) * lds, lds, w.cg, err,
+                                         timeout_ns, s);
+        if (st && st != 1) return st;
+        for (int g = 2; st == 1 && g <= kEmuSlices + 1; g++) {
             const int64_t K = (int64_t)(g - 1) * kbp;
             const uint16_t* Bg = w.sB + (col0 + j0) * lds + (int64_t)(kEmuSlices - (g - 1)) * kbp;
-            int st = launch_gemm_bf16(m, nc, K, w.sA, lds, Bg, lds, w.cg + (int64_t)(g - 2) * m * nc, m, 0, err,
-                                      timeout_ns, 0, s);
-            if (st) return st;
+            const int r = launch_gemm_bf16(m, nc, K, w.sA, lds, Bg, lds, w.cg + (int64_t)(g - 2) * m * nc, m, 0, err,
+                                           timeout_ns, 0, s);
+            if (r) return r;
         }
         k_emu_combine<<<dim3((unsigned)((m + 255) / 256), (unsigned)nc), 256, 0, s>>>(m, nc, w.cg, w.eA,
                                                                                       w.eB + col0 + j0,

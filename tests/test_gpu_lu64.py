@@ -611,3 +611,24 @@ def test_one_launch_trsm_bits(hpl, n, nb):
         hpl.lu_config(hpl.LU_TRSM_BLOCKED, 1)
     for A, ipiv in outs[1:]:
         assert torch.equal(A, outs[0][0]) and torch.equal(ipiv, outs[0][1])
+
+
+@pytest.mark.parametrize("n,nb", [(2600, 256), (2605, 192), (1030, 128), (700, 64), (701, 64), (357, 100), (130, 64)])
+def test_emulated_products_in_one_launch_bits(hpl, n, nb):
+    """The sliced update's products of few columns in one launch (look-ahead
+    columns; whole stages of K only, product columns in whole 32-column chunks,
+    either epilogue) against one launch each on wider blocks: the slice sums are
+    exact whichever way, so the factors are the same bits with the look-ahead on
+    and off, and the pivots those of the DFMA update."""
+    import torch
+    A0 = hpl.generate(19, hpl.STREAM_A, n, n)
+    outs = []
+    for emu, la in ((1, 0), (1, 1), (0, 0)):
+        A = hpl.colmajor(n, n)
+        A.copy_(A0)
+        ipiv, info = hpl.lu_factor(A, nb=nb, lookahead=la, fp64_emulation=emu)
+        torch.cuda.synchronize()
+        assert info.read()["status"] == 0
+        outs.append((A, ipiv))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    assert torch.equal(outs[0][1], outs[2][1])
