@@ -1065,7 +1065,7 @@ int launch_gemm_bf16(int64_t M, int64_t N, int64_t K, const uint16_t* A, int64_t
 // The products g = 0 .. groups - 1 of the same operands (K contiguous, groups
 // kstep of it): C_g (M x N, ld M, at C + g M N) = A(:, first (g + 1) kstep)
 // B(:, last (g + 1) kstep)^T, in one launch of the single-CTA kernel on 128 x 128
-// tiles. Returns 1 where the form does not hold: K steps that straddle a stage,
+// tiles. Returns -1 where the form does not hold: K steps that straddle a stage,
 // product columns that end inside a 32-column chunk of the epilogue, or products
 // that fill the SM pairs by themselves (the pair kernel, one launch each, is
 // faster then).
@@ -1073,11 +1073,11 @@ int launch_gemm_bf16_groups(int64_t M, int64_t N, int64_t kstep, int groups, con
                             const uint16_t* B, int64_t ldb, float* C, int* err, int64_t timeout_ns, cudaStream_t s) {
     constexpr int BN = 128, BK = tc::BKB / 2;
     const int64_t K = groups * kstep;
-    if (M <= 0 || N <= 0 || kstep <= 0 || kstep % BK || N % 32) return 1;
-    if (tc::pair_tiles(M, N, tc::tma_epilogue_ok(C, M)) || !tc::narrow_tiles(M, N)) return 1;
+    if (M <= 0 || N <= 0 || kstep <= 0 || kstep % BK || N % 32) return -1;
+    if (tc::pair_tiles(M, N, tc::tma_epilogue_ok(C, M)) || !tc::narrow_tiles(M, N)) return -1;
     const int64_t tiles = ((M + tc::BM - 1) / tc::BM) * ((N + BN - 1) / BN) * groups;
-    if (K > 0x7fffffff || N * groups > 0x7fffffff || tiles > 0x7fffffff) return 1;
-    if (lda < K || ldb < K || lda % 8 || ldb % 8 || (((uintptr_t)A | (uintptr_t)B) & 15)) return 1;
+    if (K > 0x7fffffff || N * groups > 0x7fffffff || tiles > 0x7fffffff) return -1;
+    if (lda < K || ldb < K || lda % 8 || ldb % 8 || (((uintptr_t)A | (uintptr_t)B) & 15)) return -1;
     CUtensorMap ma, mb, mc;
     int st = tc::make_map(&ma, A, M, K, lda, tc::BM, 2);
     if (st) return st;

@@ -1178,8 +1178,8 @@ static int emu_update(const LuWs& w, int64_t m, int64_t nn, int kb, int64_t col0
         const int64_t nc = std::min<int64_t>(kEmuChunk, nn - j0);
         int st = launch_gemm_bf16_groups(m, nc, kbp, kEmuSlices, w.sA, lds, w.sB + (col0 + j0) * lds, lds, w.cg, err,
                                          timeout_ns, s);
-        if (st && st != 1) return st;
-        for (int g = 2; st == 1 && g <= kEmuSlices + 1; g++) {
+        if (st > 0) return st;
+        for (int g = 2; st < 0 && g <= kEmuSlices + 1; g++) {
             const int64_t K = (int64_t)(g - 1) * kbp;
             const uint16_t* Bg = w.sB + (col0 + j0) * lds + (int64_t)(kEmuSlices - (g - 1)) * kbp;
             const int r = launch_gemm_bf16(m, nc, K, w.sA, lds, Bg, lds, w.cg + (int64_t)(g - 2) * m * nc, m, 0, err,
