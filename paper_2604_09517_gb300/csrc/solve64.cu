@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "hand_out.cuh"
 
 namespace hplgb {
 
@@ -635,10 +636,12 @@ static int solve_wave(int64_t n, const double* LU, int64_t lda, double* b, doubl
 // next tile of both is read into registers ahead of need; (d) 16 warps share
 // an SM, so the barriers of one CTA hide behind another's FMAs. The order of
 // additions into an entry does not depend on the schedule, so neither do the
-// bits. n = 4096 with 64 columns, plain and transposed solve together: 5.3 ms
+// bits. n = 4096 with 64 columns, plain and transposed solve together: 5.1 ms
 // (the FP64 rate allows 3.4), against 52 ms
 // with a diagonal and an update launch per 64 rows, one CTA on the diagonal;
-// with 2 columns a step of the chain costs 5.0 us.
+// with 2 columns a step of the chain costs 4.8 us. Each pass hands the front on
+// by hand_out's alternating words (5.2 ms with one word, which a pass that waits
+// could overwrite before the last warps had read it).
 //
 // Waits are bounded as in k_trsv_wave.
 constexpr int kMb = 32;                 // row block
@@ -678,7 +681,8 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
     double* dinv = xs + W * kMb;
     double* rhs = dinv + kMb;                         // [owned block][right-hand side][row], own thread only
     int* nj = (int*)(rhs + (size_t)R * T);            // [owned block] columns subtracted so far
-    int& s_front = nj[R];
+    int* s_front = nj + R;                            // [2] thread 0's view of the front, alternating
+    int pass = 0;
     const uint64_t deadline = globaltimer_ns() + (uint64_t)timeout_ns;
     const bool live = warp < ncol;
     double* bcol = B + (c0 + (live ? warp : 0)) * ldb;
@@ -733,7 +737,6 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
         };
 
         for (int k = t; k < R; k += T) nj[k] = 0;
-        if (t == 0) s_front = 0;
         int kp = 0, jp = 0;                            // block finished next, its next column
         int ks = R > 1 ? 1 : -1, js = 0;               // the slack's block and column
         bool xpv = false, xsv = false;                 // x of the column read ahead
@@ -863,14 +866,12 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
                     }
                 }
             }
-            if (t == 0 && P > 1) {
-                if (fnew > f && !ordered) __threadfence();   // the reads of x come after the counter's
-                s_front = fnew;
-            }
-            __syncthreads();
             if (P > 1) {
-                f = s_front;
+                if (t == 0 && fnew > f && !ordered) __threadfence();   // the reads of x come after the counter's
+                f = hand_out(s_front, pass, t == 0, fnew, [] { __syncthreads(); });
                 if (f < 0) return;
+            } else {
+                __syncthreads();
             }
         }
         __syncthreads();
@@ -910,7 +911,7 @@ static int solve_multi(int64_t n, int64_t nrhs, const double* LU, int64_t lda, d
                        int* flags, int64_t nflags, int* abort_flag, hpl_info* info, cudaStream_t s) {
     const size_t limit = wave_smem_limit();
     const int64_t nblk = (n + kMb - 1) / kMb;
-    auto bytes = [](int64_t R) { return msolve_smem_doubles(W, (int)R) * sizeof(double) + (size_t)(R + 1) * sizeof(int); };
+    auto bytes = [](int64_t R) { return msolve_smem_doubles(W, (int)R) * sizeof(double) + (size_t)(R + 2) * sizeof(int); };
     // blocks a CTA may own with 16 / W CTAs on an SM (a KB of each is reserved)
     const size_t share = limit / (16 / W) - 1024;
     if (share < bytes(1) || n > (int64_t)1 << 30) return -1;

@@ -508,6 +508,30 @@ def test_lu_solve_several_columns_zero_pivot_and_nan_column(hpl):
         assert info.read()["status_name"] == "HPL_ERR_SINGULAR"
 
 
+@pytest.mark.parametrize("nrhs,trans", [(2, 0), (2, 1), (8, 0), (16, 1)])
+def test_lu_solve_several_columns_repeats_its_bits(hpl, nrhs, trans):
+    """Solves bound by the chain of row blocks, where every CTA waits for the
+    front at nearly each step, many times over: the bits of the solve on one CTA
+    per group, which waits for nobody."""
+    import torch
+    n = 1400
+    A = hpl.generate(9, hpl.STREAM_A, n, n)
+    ipiv, _ = hpl.lu_factor(A, nb=64)
+    B0 = hpl.generate(9, hpl.STREAM_B, n, nrhs)
+    try:
+        hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, 1)
+        want = B0.clone()
+        hpl.lu_solve(A, ipiv, want, trans=trans)
+        for grid in (0, 7, 33):
+            hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, grid)
+            for _ in range(20):
+                X = B0.clone()
+                hpl.lu_solve(A, ipiv, X, trans=trans)
+                assert torch.equal(X, want)
+    finally:
+        hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, 0)
+
+
 @pytest.mark.parametrize("kind", ["uniform", "ties"])
 @pytest.mark.parametrize("n,nb,la", [(2, 64, 0), (31, 32, 0), (33, 64, 1), (65, 64, 0), (129, 40, 1), (513, 64, 0),
                                      (1100, 256, 1), (1700, 96, 1), (2200, 256, 1), (4300, 128, 1)])
