@@ -166,7 +166,19 @@ __device__ void upd64(double* A, long long lda, const double* P, int prow, int m
 // memory, combined in 64-bit integers (units 2^-58 of 2^(e(i) + e(j))) and
 // subtracted from C with one FMA. A DFMA update rounds every entry 16 times,
 // this one once, and its FP64 pipe does two operations per entry instead of
-// 16. @UPD@
+// 16: 256 uneven systems 16.2 -> 8.3 ms, 4096 64.1 -> 45.5 (8.2 and 45.1 without
+// the masks below); error of x over 600 uniform systems, median, 0.55 to 0.63 of
+// DFMA's.
+// What the cuts lose is below 2^-56.3 2^(e(i) + e(j)), whatever the entry's terms:
+// nothing beside the roundings of 16 FMAs (up to 2^-49 of sum |L||U|) when some k
+// has both its factors near their maxima, and all of it when large entries of
+// the row meet only small ones of the column (two weakly coupled blocks, say).
+// So each row of L has a mask of the k whose scaled entry is at least 2^(e - 3),
+// each column of U one of those at least 2^(e - 4): where the masks meet, sum
+// |L||U| >= 2^(e(i) + e(j) - 7) and the loss is below 2^-49.3 of it; where they
+// don't, the entry takes its 16 FMAs. Uniform systems of 128 / 512: no entry / 1.2
+// in 10^5 (with 3 bits on both sides 1.7 / 3.7 in 10^4, and a warp's share of a tile
+// meets one 7 times in 100).
 // Per 128 rows x 16 columns: the threads cut L (from the panel in shared
 // memory, once per 128 rows) and U (from global memory, fetched two tiles
 // ahead), one thread issues 8 MMAs (slice s of L against slices 1 .. 9 - s of U,
@@ -180,9 +192,9 @@ constexpr int kTcN = 16;                             // columns of a tile
 constexpr int kTcB = kTcSlices * kTcN * 16 * 2;      // 4 KB: a tile's U, two buffers
 constexpr int kTcAcc = kTcSlices * kTcN;             // TMEM columns of an accumulator, two of them
 constexpr int kTcCols = 2 * kTcAcc;
-// Smaller updates take upd64. 304 systems of 64 / 96 / 128 with the line at 16, 32,
-// 64 and 96 rows (ms): 0.254, 0.259, 0.288, 0.285 / 0.435, 0.435, 0.461, 0.547 /
-// 0.648, 0.650, 0.670, 0.757 (before the scales of k).
+// Smaller updates take upd64. 304 systems of 64 / 96 / 128 / 512 with the line at 16,
+// 32, 64 and 96 rows (ms): 0.255, 0.261, 0.278, 0.278 / 0.443, 0.445, 0.462, 0.542 /
+// 0.655, 0.661, 0.672, 0.755 / 12.26, 12.29, 12.29, 12.32: 16 and 32 do not differ.
 constexpr int kTcMinRows = 32;
 struct TcState {
     uint32_t tmem;
@@ -195,14 +207,18 @@ struct TcState {
     unsigned char* Bs;
     short* eL;              // exponents of L's rows (panel rows), U's columns (matrix columns)
     short* eU;
+    unsigned short* mU;     // U's columns: the k near the maximum (L's rows: in the panel's pad column)
     int* xk;                // [16] exponents of U's rows
 };
 
 // exponent e with every |x[k]| 2^(sgn xk) < 2^e; kTcBad outside the path's range
 constexpr int kTcBad = 30000;
 constexpr int kTcZero = -3000;      // xk of a row of zeros
+constexpr int kTcNearL = 3, kTcNearU = 4;   // bits below 2^e that count as near the maximum
 
-__device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, int sgn) {
+// near: bit k for |x[k]| 2^(sgn xk) >= 2^(e - bits); every bit where all the
+// products are zero
+__device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, int sgn, int bits, unsigned& near) {
     int mx = -100000;
     bool bad = false;
 #pragma unroll
@@ -211,17 +227,24 @@ __device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, in
         if (E) mx = max(mx, E + sgn * xk[q]);
         bad = bad || E == 0x7ff || (E == 0 && x[q] != 0.0);
     }
+    near = 0xffffu;
     if (bad) return kTcBad;
     if (mx < -1000) return 0;       // zeros, or only entries that meet rows of zeros
+    near = 0;
+#pragma unroll
+    for (int q = 0; q < 16; q++) {
+        const int E = tc::expo(x[q]);
+        if (E && E + sgn * xk[q] > mx - bits) near |= 1u << q;
+    }
     return mx < 1022 - 400 || mx > 1022 + 400 ? kTcBad : mx - 1022;
 }
 
 // The scales of a panel: xk from U's rows, then eL (panel rows prow ..) and eU
-// (columns c1 .. n). Nonzero: this thread met something outside the range. Each
+// (columns c1 .. n), and the masks beside them. Nonzero: this thread met something outside the range. Each
 // thread holds its two columns of U across the reduction (n <= 512). Not
 // inlined, as upd_tc.
-__device__ __noinline__ int tc_levels(const double* A, long long lda, const double* P, int prow, int n, int c1, int k0,
-                                      short* eL, short* eU, int* xk) {
+__device__ __noinline__ int tc_levels(const double* A, long long lda, double* P, int prow, int n, int c1, int k0,
+                                      short* eL, short* eU, unsigned short* mU, int* xk) {
     static_assert(NMAX <= 2 * THREADS, "two columns per thread");
     double u[2][16];
     int bad = 0;
@@ -249,17 +272,21 @@ __device__ __noinline__ int tc_levels(const double* A, long long lda, const doub
     for (int h = 0; h < 2; h++) {
         const int c = c1 + threadIdx.x + h * THREADS;
         if (c >= n) continue;
-        const int e = tc_level(u[h], xk, -1);
+        unsigned near;
+        const int e = tc_level(u[h], xk, -1, kTcNearU, near);
         bad |= e == kTcBad;
         eU[c] = (short)e;
+        mU[c] = (unsigned short)near;
     }
     for (int r = prow + threadIdx.x; r < n - k0; r += THREADS) {
         double x[16];
 #pragma unroll
         for (int q = 0; q < 16; q++) x[q] = P[r * panel_stride<16>() + q];
-        const int e = tc_level(x, xk, 1);
+        unsigned near;
+        const int e = tc_level(x, xk, 1, kTcNearL, near);
         bad |= e == kTcBad;
         eL[r] = (short)e;
+        *reinterpret_cast<unsigned*>(P + r * panel_stride<16>() + 16) = near;
     }
     return bad;
 }
@@ -291,6 +318,28 @@ __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
                  : "memory");
+}
+
+// nonzero where a 16-bit half of x is zero; the zero halves of x as 8 bits
+__device__ __forceinline__ unsigned tc_zero_half(unsigned x) { return (x - 0x10001u) & ~x & 0x80008000u; }
+__device__ __forceinline__ unsigned tc_zero_halves(uint4 x) {
+    const unsigned w[4] = {x.x, x.y, x.z, x.w};
+    unsigned r = 0;
+#pragma unroll
+    for (int q = 0; q < 4; q++) r |= ((w[q] & 0xffffu) == 0) << (2 * q) | ((w[q] >> 16) == 0) << (2 * q + 1);
+    return r;
+}
+
+// The entries cp[j ld] of one row, j a bit of cols, by FMAs: l the row of L, u the
+// columns of U.
+__device__ __noinline__ void upd_fma(double* cp, long long ld, const double* u, const double* l, unsigned cols) {
+    for (; cols; cols &= cols - 1) {
+        const int j = __ffs(cols) - 1;
+        double x = cp[j * ld];
+#pragma unroll
+        for (int q = 0; q < 16; q++) x = fma(-l[q], u[j * ld + q], x);
+        cp[j * ld] = x;
+    }
 }
 
 // C (rows r0.., columns c0.., m x m) -= L (panel rows prow..) U (global rows
@@ -347,6 +396,8 @@ __device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* 
         cut_u(0);
         const bool rin = ti + frow < m;
         const int eL = rin ? tc.eL[prow + ti + frow] : 0;
+        const double* const prw = P + (prow + ti + frow) * panel_stride<16>();
+        const unsigned mL = rin ? *reinterpret_cast<const unsigned*>(prw + 16) * 0x10001u : ~0u;
         double cv[8];
         double* const crow = A + (c0 + 8 * half) * lda + r0 + ti + frow;
         auto width = [&](int t) { return rin ? min(8, m - t * kTcN - 8 * half) : 0; };
@@ -384,13 +435,23 @@ __device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* 
             if (t > 0) {
                 const int f = t - 1;
                 const uint32_t a = (tc.tiles + f) & 1u;
+                const int nc = width(f);
+                double* cp = crow + (long long)f * kTcN * lda;
+                // columns whose mask and this row's don't meet (c0 is a multiple of 16):
+                // beside the MMAs
+                const uint4 mU = *reinterpret_cast<const uint4*>(tc.mU + c0 + f * kTcN + 8 * half);
+                const uint4 mm = make_uint4(mU.x & mL, mU.y & mL, mU.z & mL, mU.w & mL);
+                unsigned live = nc > 0 ? (1u << nc) - 1 : 0u;
+                if (tc_zero_half(mm.x) | tc_zero_half(mm.y) | tc_zero_half(mm.z) | tc_zero_half(mm.w)) {
+                    const unsigned apart = live & tc_zero_halves(mm);
+                    if (apart) upd_fma(cp, lda, A + (c0 + f * kTcN + 8 * half) * lda + k0, prw, apart);
+                    live &= ~apart;
+                }
                 const bool ok = tc::mbar_wait(&tc.bar[a], ((tc.tiles + f) >> 1) & 1u, tc.deadline, tc.abort, tc.err);
                 if (!__all_sync(0xffffffffu, ok)) *tc.abort = 1;
                 tc::tc_fence_after();
                 cut_u(t + 1);                              // tile t - 1's slices have been read
                 const uint32_t ta = tc.tmem + ((uint32_t)((warp & 3) * 32) << 16) + a * kTcAcc + half * 8;
-                const int nc = width(f);
-                double* cp = crow + (long long)f * kTcN * lda;
                 const short* eU = tc.eU + c0 + f * kTcN + 8 * half;
 #pragma unroll
                 for (int j4 = 0; j4 < 2; j4++) {
@@ -409,7 +470,7 @@ __device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* 
                         const long long lo = (long long)two(4) * 65536 + two(6);       // units 2^-72
                         const long long v = hi * (1 << 18) + (lo >> 14);               // units 2^-58
                         const double scale = __longlong_as_double((long long)(eL + eU[jj] - 58 + 1023) << 52);
-                        if (jj < nc) cp[jj * lda] = fma(-(double)v, scale, cv[jj]);
+                        if (live >> jj & 1u) cp[jj * lda] = fma(-(double)v, scale, cv[jj]);
                     }
                 }
             }
@@ -604,7 +665,7 @@ __device__ bool lu64(const Sys& S, double* P, double* Us, long long* redk, long 
             if constexpr (NB == 16)
                 if (use_tc) {
                     __syncthreads();
-                    bad = tc_levels(A, lda, P, kb, n, c1, k0, tc.eL, tc.eU, tc.xk);
+                    bad = tc_levels(A, lda, P, kb, n, c1, k0, tc.eL, tc.eU, tc.mU, tc.xk);
                 }
             if (use_tc && !__syncthreads_or(bad)) {
                 tc.tiles = upd_tc(A, lda, P, kb, m, c1, c1, k0, tc);
@@ -961,13 +1022,13 @@ __device__ void mxp_one(const Sys& S, const Header* H, float* X, float* R, float
 
 // Dynamic shared memory of a run whose widest panel is NBR: the FP64 panel
 // (NMAX x (NBR + 1)), the U block (NBR x 65; the slices of U for upd_tc), three
-// NBR x NBR FP32 blocks (the exponents for upd_tc), the slices of L.
+// NBR x NBR FP32 blocks (the exponents and masks for upd_tc), the slices of L.
 template <int NBR>
 constexpr size_t smem_bytes() {
     return sizeof(double) * (NMAX * panel_stride<NBR>() + NBR * 65) + sizeof(float) * 3 * NBR * NBR + kTcA;
 }
-static_assert(sizeof(double) * 16 * 65 >= 2 * kTcB && sizeof(float) * 3 * 16 * 16 >= 2 * sizeof(short) * NMAX,
-              "upd_tc's slices of U and exponents share the buffers of the other paths");
+static_assert(sizeof(double) * 16 * 65 >= 2 * kTcB && sizeof(float) * 3 * 16 * 16 >= 3 * sizeof(short) * NMAX,
+              "upd_tc's slices of U, exponents and masks share the buffers of the other paths");
 
 }  // namespace bt
 
@@ -1216,7 +1277,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
     __syncthreads();
     tc::tc_fence_after();
     TcState tc{s_tmem, s_bar, 0u, 0, &s_abort, &s_err, (unsigned char*)(T + NBR * NBR), (unsigned char*)Us, (short*)X,
-               (short*)X + NMAX, s_xk};
+               (short*)X + NMAX, (unsigned short*)X + 2 * NMAX, s_xk};
     const int pref = s_pref;
     const int lo[2] = {0, H->count0}, sz[2] = {H->count0, H->count - H->count0};
     for (;;) {

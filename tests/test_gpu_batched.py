@@ -269,3 +269,38 @@ def test_batched_update_range(hpl):
     R = np.abs(A0[3][perm] - (np.tril(LU, -1) + np.eye(m)) @ np.triu(LU))
     assert (R <= m * 2.0 ** -1074 + m * EPS * (np.abs(np.tril(LU, -1) + np.eye(m)) @ np.abs(np.triu(LU)))).all()
     assert not np.isfinite(_np(bt.matrix(6))).all() and np.isinf(_np(bt.matrix(6))).any()
+
+
+def _weakly_coupled(n, e, seed):
+    """Two uniform blocks with interleaved unknowns, their coupling 2^-e in size
+    (none at all for e = 0)."""
+    r = np.random.default_rng(seed)
+    i = np.arange(n)
+    weak = 2.0 ** -e if e else 0.0
+    return r.uniform(-0.5, 0.5, (n, n)) * np.where((i[:, None] + i) % 2, weak, 1.0)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+def test_batched_update_keeps_small_terms(hpl, variant):
+    """Large entries of a row of L that meet only small ones of a column of U:
+    interleaved blocks of weak (and no) coupling, a single entry 2^50 above the
+    rest, rows and columns graded against each other. The bound of an LU made of
+    rounded products holds entry by entry with either panel width."""
+    import torch
+    mats = [_weakly_coupled(n, e, 100 * n + e) for n in (96, 200) for e in (0, 20, 30, 40, 50, 100)]
+    spike = np.random.default_rng(7).uniform(-0.5, 0.5, (160, 160))
+    spike[90, 30] = 2.0 ** 50
+    g = np.arange(120)
+    graded = np.random.default_rng(8).uniform(-0.5, 0.5, (120, 120)) * 2.0 ** -np.abs(g[:, None] - g).astype(float)
+    mats += [spike, graded]
+    n = np.array([len(m) for m in mats], dtype=np.int64)
+    bt = hpl.Batch(n, np.zeros(len(n), dtype=np.uint8))
+    bt.B.fill_(1.0)
+    for s, m in enumerate(mats):
+        bt.matrix(s).copy_(torch.from_numpy(m).cuda())
+    bt.plan(variant=variant)
+    bt.run()
+    torch.cuda.synchronize()
+    for s, m in enumerate(mats):
+        assert bt.info(s)["status"] == 0
+        assert _backward_error_bound_holds(m, _np(bt.matrix(s)), _np(bt.pivots(s))), s
