@@ -14,11 +14,19 @@
 //    memory: over 256 k at most 11 * 256 products below 2^12, so every partial
 //    sum is an integer below 2^24 and exact. After each 256 k the 11 sums move
 //    into two 64-bit integers per entry, exactly; one rounding to FP64 at the
-//    end of the K slice. What is lost is below 2^-62 of (row maximum) * (column
-//    maximum) per term, against 2^-53 of every term and partial sum in FP64
-//    arithmetic.
-//  * Infinities and NaN: a row of A or a column of B that holds one gives NaN.
-//    Subnormal entries count as zero.
+//    end of the K slice. What is lost is below 2^-61.8 2^(eA + eB) per term, with
+//    2^eA and 2^eB the powers of two above the row's and the column's maximum.
+//  * FP64 arithmetic loses up to 2^-53 of sum |a||b| per term, which is far less
+//    when the large entries of the row meet only small ones of the column (two
+//    weakly coupled groups of unknowns, gradients that vanish where X is large).
+//    So an entry is taken from the slices only where sum |a||b| is at least
+//    2^(eA + eB - 8.7), where they lose no more than K roundings of FP64. The sums
+//    of the slice products over 256 k, added without their signs, bound it from
+//    below and settle that for nearly every entry (kEnough). The rest is looked at
+//    by FMAs (by_fma), which also form the entries that the slices must not: dense
+//    operands keep the slices' bits.
+//  * Rows of A and columns of B with an infinity, a NaN or a subnormal entry
+//    take FMAs as well.
 //
 // One CTA computes 128 rows x 32 columns over one K slice:
 //   warps 0-15: two groups of 8 that take the stages in turn. Each thread
@@ -51,6 +59,11 @@ namespace p64 {
 
 using namespace tc;
 
+// not 0, with an exponent field of 0
+__device__ __forceinline__ bool subnormal(double v) {
+    return expo(v) == 0 && ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) != 0;
+}
+
 constexpr int kSlices = 11;
 constexpr int kRows = 128, kCols = 32, kStep = 16;         // a CTA's tile, k per stage
 constexpr int kChunk = 256 / kStep;                        // stages between folds
@@ -63,7 +76,9 @@ constexpr int kSmem = kStages * (kAStage + kBStage) + kRaw;
 constexpr int kThreads = kProducers + 32;
 constexpr int64_t kMaxSlice = 65536;                       // k per CTA: the low 64-bit sums hold 512 chunks
 constexpr int kNoScale = -4000;                            // xk of a zero row of B
-constexpr int kBad = 1 << 24;                              // eB of a column with an infinity or NaN
+constexpr int kBad = 1 << 24;                              // eB of a column with an infinity, a NaN or a subnormal
+constexpr int kLow = -(1 << 20);                           // exponent of a row or column of zeros
+constexpr unsigned kEnough = 255;                          // sum |a||b| in units of 2^(eA + eB - 12) / 26, saturated: 2^-8.7
 
 // The 11 slices of 8 consecutive k as 8 BF16 values each (k ascending), handed
 // to put(slice, uint4), from the fixed-point magnitudes T and the signs (bit q
@@ -131,22 +146,24 @@ __global__ void __launch_bounds__(128) k_scale_k(int64_t nn, const double* __res
     if (threadIdx.x == 0) xk[blockIdx.x] = mx ? mx - 1022 : kNoScale;
 }
 
-// eB[c] = e with every |B(., c)| 2^-xk < 2^e (kBad: an infinity or NaN); one CTA per c
+// eB[c] = e with every |B(., c)| 2^-xk < 2^e (kBad: an infinity, a NaN or a
+// subnormal; kLow: zeros); one CTA per c
 __global__ void __launch_bounds__(128) k_scale_c(int64_t K, const double* __restrict__ B, int64_t sk, int64_t sc,
                                                  const int* __restrict__ xk, int* __restrict__ eB) {
     __shared__ int s[4];
     const double* b = B + (int64_t)blockIdx.x * sc;
-    int mx = -(1 << 20);
+    int mx = kLow;
     for (int64_t k = threadIdx.x; k < K; k += 128) {
-        const int E = expo(b[k * sk]);
-        if (E == 0x7ff) mx = kBad;
+        const double v = b[k * sk];
+        const int E = expo(v);
+        if (E == 0x7ff || subnormal(v)) mx = kBad;
         else if (E) mx = max(mx, E - xk[k]);
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mx;
     __syncthreads();
     mx = max(max(s[0], s[1]), max(s[2], s[3]));
-    if (threadIdx.x == 0) eB[blockIdx.x] = mx == kBad ? kBad : mx < -(1 << 19) ? 0 : mx - 1022;
+    if (threadIdx.x == 0) eB[blockIdx.x] = mx == kBad || mx == kLow ? mx : mx - 1022;
 }
 
 // The image of B: per 32 columns, per 16 k: [k octet][slice][group of 8
@@ -162,7 +179,7 @@ __global__ void __launch_bounds__(256) k_slice_b(int64_t K, int64_t nn, const do
     const int64_t oct = t / kCols % octs, g = t / (kCols * octs), c = g * kCols + cl, k0 = 8 * oct;
     unsigned long long T[8];
     unsigned sgn = 0;
-    const int e = c < nn ? eB[c] : 0;
+    const int e = c < nn ? eB[c] : kBad;
 #pragma unroll
     for (int q = 0; q < 8; q++) {
         const bool in = c < nn && k0 + q < K && e != kBad;
@@ -184,9 +201,9 @@ __device__ __forceinline__ void mma_n(uint32_t d, uint64_t a, uint64_t b, int N,
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
                  : "memory");
 }
@@ -196,13 +213,92 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src, bool vali
                  "r"(valid ? BYTES : 0) : "memory");
 }
 
+// The entries of a warp's 32 rows from r0 (lane l: row r0 + l) and columns c0 + j
+// that have a bit j in which: sum a b and sum |a||b| by FMAs over the k of [ka, kb),
+// the first into out[j ldc] unless the second reaches 0.6 2^(eA + eB - 8) (eA: the
+// lane's; kBad in either: never), where the slices' entry stays. A column's
+// entries are formed side by side, a lane each (lanes read neighbours of A), or,
+// when few of them are wanted or A's rows lie along memory (TA), one after the
+// other by all lanes along k. Many entries of one column over several times 256 k
+// are no chance cancellations: sum |a||b|, half the FMAs, is then left out. n = 4096
+// with 64 columns, every second unknown coupled by 2^-40, forward and backward:
+// 21.7 ms (17.4 with DFMA kernels throughout, 4.9 uniform).
+template <bool TA>
+__device__ __noinline__ void by_fma(unsigned which, const double* A, int64_t lda, int64_t r0, int64_t M, int eA,
+                                    const double* B, int64_t sk, int64_t sc, int64_t c0, const int* eB, int64_t ka,
+                                    int64_t kb, double* out, int64_t ldc, int neg) {
+    const int lane = threadIdx.x & 31;
+    for (int j = 0; j < 8; j++) {
+        const bool mine = which >> j & 1u;
+        unsigned m = __ballot_sync(0xffffffffu, mine);
+        if (!m) continue;
+        const double* b = B + (c0 + j) * sc;
+        const int ec = eB[c0 + j];
+        const double enough = eA == kBad || ec == kBad ? __longlong_as_double(0x7ff8000000000000LL) : ldexp(0.6, eA + ec - 8);
+        const bool many = __popc(m) > 4, weigh = !many || kb - ka <= 256;
+        if (!TA && many) {
+            const double* a = A + min(r0 + lane, M - 1);
+            double s[2] = {0.0, 0.0}, t[2] = {0.0, 0.0};
+            for (int64_t k = ka; k < kb; k += 8) {
+                double x[8], y[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    x[u] = k + u < kb ? a[(k + u) * lda] : 0.0;
+                    y[u] = k + u < kb ? b[(k + u) * sk] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; u++) s[u & 1] = fma(x[u], y[u], s[u & 1]);
+                if (!weigh) continue;
+#pragma unroll
+                for (int u = 0; u < 8; u++) t[u & 1] = fma(fabs(x[u]), fabs(y[u]), t[u & 1]);
+                if (!__any_sync(0xffffffffu, mine && !(t[0] + t[1] >= enough))) break;
+            }
+            const double v = s[0] + s[1];
+            if (mine && !(weigh && t[0] + t[1] >= enough)) out[j * ldc] = neg ? -v : v;
+            continue;
+        }
+        for (; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const double* a = TA ? A + (r0 + l) * lda : A + r0 + l;
+            const int64_t step = TA ? 1 : lda;
+            const double lim = __shfl_sync(0xffffffffu, enough, l), per = 65536.0 / lim;
+            double s = 0.0, t = 0.0;
+            bool keep = false;                                 // the slices' entry
+            for (int64_t k0 = ka; k0 < kb && !keep; k0 += 128) {
+                double x[4], y[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int64_t k = k0 + 32 * u + lane;
+                    x[u] = k < kb ? a[k * step] : 0.0;
+                    y[u] = k < kb ? b[k * sk] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) s = fma(x[u], y[u], s);
+                if (!weigh) continue;
+#pragma unroll
+                for (int u = 0; u < 4; u++) t = fma(fabs(x[u]), fabs(y[u]), t);
+                // the lanes' shares in units of 2^-16 lim, rounded down
+                keep = lim == lim && __reduce_add_sync(0xffffffffu, (unsigned)fmin(t * per, 65536.0)) >= 65536u;
+            }
+            if (keep) continue;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, off);
+                t += __shfl_xor_sync(0xffffffffu, t, off);
+            }
+            if (lane == l && !(weigh && t >= lim)) out[j * ldc] = neg ? -s : s;
+        }
+    }
+}
+
 // C(z) (M x nn, ld ldc, slice z at C + z zstride) = (neg ? - : +) op(A) B over
 // the k of slice z, [z kslice, (z + 1) kslice); kslice a multiple of 16.
 // op(A)(i, k) = A[k lda + i], or A[i lda + k] (TA).
 template <bool TA>
 __global__ void __launch_bounds__(kThreads, 1)
 k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restrict__ A, int64_t lda, int vec,
-         const unsigned char* __restrict__ img, const int* __restrict__ xk, const int* __restrict__ eB,
+         const double* __restrict__ B, int64_t sk, int64_t sc, const unsigned char* __restrict__ img,
+         const int* __restrict__ xk, const int* __restrict__ eB,
          double* __restrict__ C, int64_t ldc, int64_t zstride, int neg, int* err, int64_t timeout_ns) {
     extern __shared__ __align__(1024) unsigned char psm[];
     __shared__ __align__(8) uint64_t full[kStages], bfull[kStages], empty[kStages], accfull, accempty, drain;
@@ -215,7 +311,6 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
     const int nst = (int)((kb - ka + kStep - 1) / kStep);          // >= 1
     const int nch = (nst + kChunk - 1) / kChunk;
     const uint64_t deadline = globaltimer_ns() + (uint64_t)timeout_ns;
-    constexpr int kLow = -(1 << 20);                               // exponent of a row of zeros
     if (tid == 0) {
         s_abort = 0;
         for (int s = 0; s < kStages; s++) {
@@ -236,7 +331,7 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
         // the rows' largest exponents over this K slice, many loads in flight
         auto level = [&](double v, int x) {
             const int E = expo(v);
-            return E == 0x7ff ? kBad : E ? E + x : kLow;
+            return E == 0x7ff || subnormal(v) ? kBad : E ? E + x : kLow;
         };
         if (TA) {
             for (int i = 0; i < kRows / 16; i += 2) {              // two rows at a time
@@ -301,10 +396,10 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
             mbar_wait(&drain, 0, deadline + 1000000000ull, &s_abort, err);
         }
     } else {
-        // the exponent of local row r (0 for a row of zeros, kBad kept)
+        // the exponent of local row r (kLow where it meets only zeros, kBad kept)
         auto row_exp = [&](int r) {
             const int mx = max(max(s_e[0][r], s_e[1][r]), max(s_e[2][r], s_e[3][r]));
-            return mx >= kBad ? kBad : mx == kLow ? 0 : mx - 1022;
+            return mx >= kBad ? kBad : mx < kNoScale / 2 ? kLow : mx - 1022;
         };
         const int grp = warp >> 3;                                  // takes stages grp, grp + 2, ...
         const int row = tid & (kRows - 1), oct = (tid >> 7) & 1;    // as a producer
@@ -312,6 +407,7 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
         const bool rowin = r0 + row < M && e != kBad;
         const int quarter = warp >> 2;                              // as a folder: row 32 (warp & 3) + lane,
         long long hi[8], lo[8];                                     // columns 8 quarter + j
+        unsigned size[2] = {0u, 0u};                                // the like of all k, a byte per column
 #pragma unroll
         for (int j = 0; j < 8; j++) hi[j] = lo[j] = 0;
         // this thread's next 8 values of A: pairs (2q, 2q + 1) at raw[q * kProducers + tid]
@@ -347,15 +443,30 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
             tc_fence_after();
             const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16) + quarter * 8;
 #pragma unroll
-            for (int g = 0; g < kSlices; g++) {
-                uint32_t r[8];
-                tmem_ld8(ta + g * kCols, r);
-                tmem_wait_ld();
+            for (int h = 0; h < 2; h++) {
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};                // bounds sum |a||b| of these 256 k, units 2^-12
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const int iv = __float2int_rn(__uint_as_float(r[j]));
-                    if (g < 5) hi[j] += (long long)iv * (1 << (6 * (4 - g)));    // units 2^-36
-                    else lo[j] += (long long)iv * (1 << (6 * (10 - g)));         // units 2^-72
+                for (int g = 0; g < kSlices; g++) {
+                    uint32_t r[4];
+                    tmem_ld4(ta + g * kCols + 4 * h, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int jj = 0; jj < 4; jj++) {
+                        const int j = 4 * h + jj;
+                        const float f = __uint_as_float(r[jj]);
+                        const int iv = __float2int_rn(f);
+                        if (g < 5) {
+                            hi[j] += (long long)iv * (1 << (6 * (4 - g)));       // units 2^-36
+                            sum[jj] = fmaf(fabsf(f), 1.0f / (1 << (6 * g)), sum[jj]);
+                        } else {
+                            lo[j] += (long long)iv * (1 << (6 * (10 - g)));      // units 2^-72
+                        }
+                    }
+                }
+#pragma unroll
+                for (int jj = 0; jj < 4; jj++) {
+                    const unsigned q = min((unsigned)(sum[jj] * 26.0f), kEnough);
+                    size[h] = __vaddus4(size[h], q << (8 * jj));
                 }
             }
             tc_fence_before();
@@ -410,8 +521,9 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
         if (ok) {
             const int fr = (warp & 3) * 32 + lane, fe = row_exp(fr);
             const int64_t r = r0 + fr;
+            double* out = C + (int64_t)blockIdx.z * zstride + min(r, M - 1);
+            unsigned again = 0;                                     // columns whose entry may not be the slices'
             if (r < M) {
-                double* out = C + (int64_t)blockIdx.z * zstride + r;
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
                     const int64_t c = c0 + 8 * quarter + j;
@@ -420,10 +532,15 @@ k_prod64(int64_t M, int64_t nn, int64_t K, int64_t kslice, const double* __restr
                     double v = fma((double)lo[j], 0x1p-36, (double)hi[j]);
                     const int ex = fe + ec - 36;
                     v = ex > -1022 && ex < 1024 ? v * __longlong_as_double((long long)(ex + 1023) << 52) : ldexp(v, ex);
-                    if (fe == kBad || ec == kBad) v = __longlong_as_double(0x7ff8000000000000LL);
+                    if (fe == kBad || ec == kBad ||
+                        (fe != kLow && ec != kLow && (size[j >> 2] >> (8 * (j & 3)) & 255u) < kEnough))
+                        again |= 1u << j;
                     out[c * ldc] = neg ? -v : v;
                 }
             }
+            const int64_t c = c0 + 8 * quarter;
+            if (__any_sync(0xffffffffu, again != 0))
+                by_fma<TA>(again, A, lda, r0 + (warp & 3) * 32, M, fe, B, sk, sc, c, eB, ka, kb, out + c * ldc, ldc, neg);
         }
     }
     tc_fence_before();
@@ -475,8 +592,8 @@ int launch_prod64(int64_t M, int64_t nn, int64_t K, int ta, const double* A, int
     k_slice_b<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(K, nn, B, sk, sc, xk, eB, img);
     HPL_LAUNCH_CHECK();
     const dim3 g((unsigned)rt, (unsigned)cg, (unsigned)split);
-    if (ta) k_prod64<true><<<g, kThreads, kSmem, s>>>(M, nn, K, kslice, A, lda, vec, img, xk, eB, C, ldc, zstride, neg, err, timeout_ns);
-    else k_prod64<false><<<g, kThreads, kSmem, s>>>(M, nn, K, kslice, A, lda, vec, img, xk, eB, C, ldc, zstride, neg, err, timeout_ns);
+    if (ta) k_prod64<true><<<g, kThreads, kSmem, s>>>(M, nn, K, kslice, A, lda, vec, B, sk, sc, img, xk, eB, C, ldc, zstride, neg, err, timeout_ns);
+    else k_prod64<false><<<g, kThreads, kSmem, s>>>(M, nn, K, kslice, A, lda, vec, B, sk, sc, img, xk, eB, C, ldc, zstride, neg, err, timeout_ns);
     HPL_LAUNCH_CHECK();
     return HPL_OK;
 }
