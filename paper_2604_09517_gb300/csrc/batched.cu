@@ -166,19 +166,20 @@ __device__ void upd64(double* A, long long lda, const double* P, int prow, int m
 // memory, combined in 64-bit integers (units 2^-58 of 2^(e(i) + e(j))) and
 // subtracted from C with one FMA. A DFMA update rounds every entry 16 times,
 // this one once, and its FP64 pipe does two operations per entry instead of
-// 16: 256 uneven systems 16.2 -> 8.3 ms, 4096 64.1 -> 45.5 (8.2 and 45.1 without
+// 16: 256 uneven systems 16.2 -> 8.0 ms, 4096 64.1 -> 44.0 (8.2 and 44.5 without
 // the masks below); error of x over 600 uniform systems, median, 0.55 to 0.63 of
 // DFMA's.
 // What the cuts lose is below 2^-56.3 2^(e(i) + e(j)), whatever the entry's terms:
 // nothing beside the roundings of 16 FMAs (up to 2^-49 of sum |L||U|) when some k
 // has both its factors near their maxima, and all of it when large entries of
 // the row meet only small ones of the column (two weakly coupled blocks, say).
-// So each row of L has a mask of the k whose scaled entry is at least 2^(e - 3),
-// each column of U one of those at least 2^(e - 4): where the masks meet, sum
-// |L||U| >= 2^(e(i) + e(j) - 7) and the loss is below 2^-49.3 of it; where they
-// don't, the entry takes its 16 FMAs. Uniform systems of 128 / 512: no entry / 1.2
-// in 10^5 (with 3 bits on both sides 1.7 / 3.7 in 10^4, and a warp's share of a tile
-// meets one 7 times in 100).
+// Each row of L has masks of the k whose scaled entry is at least 2^(e - 3) and
+// 2^(e - 4), each column of U one of those at least 2^(e - 4). Where the first meets
+// the column's, or the second does in two places, sum |L||U| >= 2^(e(i) + e(j) - 7)
+// and the loss is below 2^-49.3 of it; otherwise that sum is formed and the entry
+// takes its 16 FMAs if it is smaller. Uniform systems keep the slices' bits: of 512
+// rows 1.2 entries in 10^5 come to the second mask (with 3 bits on both sides 3.7
+// in 10^4, and a warp's share of a tile meets one 7 times in 100).
 // Per 128 rows x 16 columns: the threads cut L (from the panel in shared
 // memory, once per 128 rows) and U (from global memory, fetched two tiles
 // ahead), one thread issues 8 MMAs (slice s of L against slices 1 .. 9 - s of U,
@@ -214,11 +215,11 @@ struct TcState {
 // exponent e with every |x[k]| 2^(sgn xk) < 2^e; kTcBad outside the path's range
 constexpr int kTcBad = 30000;
 constexpr int kTcZero = -3000;      // xk of a row of zeros
-constexpr int kTcNearL = 3, kTcNearU = 4;   // bits below 2^e that count as near the maximum
+constexpr int kTcNear = 3;          // bits below 2^e that count as near the maximum (and one more)
 
-// near: bit k for |x[k]| 2^(sgn xk) >= 2^(e - bits); every bit where all the
-// products are zero
-__device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, int sgn, int bits, unsigned& near) {
+// near: bit k for |x[k]| 2^(sgn xk) >= 2^(e - kTcNear), bit k + 16 for twice as far
+// down; every bit where all the products are zero
+__device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, int sgn, unsigned& near) {
     int mx = -100000;
     bool bad = false;
 #pragma unroll
@@ -227,14 +228,15 @@ __device__ __forceinline__ int tc_level(const double (&x)[16], const int* xk, in
         if (E) mx = max(mx, E + sgn * xk[q]);
         bad = bad || E == 0x7ff || (E == 0 && x[q] != 0.0);
     }
-    near = 0xffffu;
+    near = ~0u;
     if (bad) return kTcBad;
     if (mx < -1000) return 0;       // zeros, or only entries that meet rows of zeros
     near = 0;
 #pragma unroll
     for (int q = 0; q < 16; q++) {
         const int E = tc::expo(x[q]);
-        if (E && E + sgn * xk[q] > mx - bits) near |= 1u << q;
+        const int d = E ? mx - E - sgn * xk[q] : 99;
+        near |= (d < kTcNear ? 0x10001u : d == kTcNear ? 0x10000u : 0u) << q;
     }
     return mx < 1022 - 400 || mx > 1022 + 400 ? kTcBad : mx - 1022;
 }
@@ -273,17 +275,17 @@ __device__ __noinline__ int tc_levels(const double* A, long long lda, double* P,
         const int c = c1 + threadIdx.x + h * THREADS;
         if (c >= n) continue;
         unsigned near;
-        const int e = tc_level(u[h], xk, -1, kTcNearU, near);
+        const int e = tc_level(u[h], xk, -1, near);
         bad |= e == kTcBad;
         eU[c] = (short)e;
-        mU[c] = (unsigned short)near;
+        mU[c] = (unsigned short)(near >> 16);
     }
     for (int r = prow + threadIdx.x; r < n - k0; r += THREADS) {
         double x[16];
 #pragma unroll
         for (int q = 0; q < 16; q++) x[q] = P[r * panel_stride<16>() + q];
         unsigned near;
-        const int e = tc_level(x, xk, 1, kTcNearL, near);
+        const int e = tc_level(x, xk, 1, near);
         bad |= e == kTcBad;
         eL[r] = (short)e;
         *reinterpret_cast<unsigned*>(P + r * panel_stride<16>() + 16) = near;
@@ -320,26 +322,39 @@ __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                  : "memory");
 }
 
-// nonzero where a 16-bit half of x is zero; the zero halves of x as 8 bits
+// nonzero where a 16-bit half of x is zero
 __device__ __forceinline__ unsigned tc_zero_half(unsigned x) { return (x - 0x10001u) & ~x & 0x80008000u; }
-__device__ __forceinline__ unsigned tc_zero_halves(uint4 x) {
-    const unsigned w[4] = {x.x, x.y, x.z, x.w};
+
+// columns (a bit each) whose mask does not meet a row's masks nL as it should
+__device__ __forceinline__ unsigned tc_apart(uint4 mU, unsigned nL) {
+    const unsigned w[4] = {mU.x, mU.y, mU.z, mU.w};
     unsigned r = 0;
 #pragma unroll
-    for (int q = 0; q < 4; q++) r |= ((w[q] & 0xffffu) == 0) << (2 * q) | ((w[q] >> 16) == 0) << (2 * q + 1);
+    for (int j = 0; j < 8; j++) {
+        const unsigned m = w[j >> 1] >> (16 * (j & 1)) & 0xffffu, far = m & nL >> 16;
+        if (!(m & nL) && !(far & (far - 1))) r |= 1u << j;
+    }
     return r;
 }
 
-// The entries cp[j ld] of one row, j a bit of cols, by FMAs: l the row of L, u the
-// columns of U.
-__device__ __noinline__ void upd_fma(double* cp, long long ld, const double* u, const double* l, unsigned cols) {
+// The entries cp[j ld] of one row, j a bit of cols, by FMAs where sum |L||U| is
+// below 2^(eL + eU[j] - 7): l the row of L, u the columns of U. Returns their bits.
+__device__ __noinline__ unsigned upd_fma(double* cp, long long ld, const double* u, const double* l, unsigned cols,
+                                         int eL, const short* eU) {
+    unsigned done = 0;
     for (; cols; cols &= cols - 1) {
         const int j = __ffs(cols) - 1;
+        double s = 0.0;
+#pragma unroll 2
+        for (int q = 0; q < 16; q++) s = fma(fabs(l[q]), fabs(u[j * ld + q]), s);
+        if (s >= __longlong_as_double((long long)(eL + eU[j] - 7 + 1023) << 52)) continue;
         double x = cp[j * ld];
-#pragma unroll
+#pragma unroll 2
         for (int q = 0; q < 16; q++) x = fma(-l[q], u[j * ld + q], x);
         cp[j * ld] = x;
+        done |= 1u << j;
     }
+    return done;
 }
 
 // C (rows r0.., columns c0.., m x m) -= L (panel rows prow..) U (global rows
@@ -397,7 +412,7 @@ __device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* 
         const bool rin = ti + frow < m;
         const int eL = rin ? tc.eL[prow + ti + frow] : 0;
         const double* const prw = P + (prow + ti + frow) * panel_stride<16>();
-        const unsigned mL = rin ? *reinterpret_cast<const unsigned*>(prw + 16) * 0x10001u : ~0u;
+        const unsigned nL = rin ? *reinterpret_cast<const unsigned*>(prw + 16) : ~0u, mL = (nL & 0xffffu) * 0x10001u;
         double cv[8];
         double* const crow = A + (c0 + 8 * half) * lda + r0 + ti + frow;
         auto width = [&](int t) { return rin ? min(8, m - t * kTcN - 8 * half) : 0; };
@@ -437,22 +452,21 @@ __device__ __noinline__ uint32_t upd_tc(double* A, long long lda, const double* 
                 const uint32_t a = (tc.tiles + f) & 1u;
                 const int nc = width(f);
                 double* cp = crow + (long long)f * kTcN * lda;
+                const short* eU = tc.eU + c0 + f * kTcN + 8 * half;
                 // columns whose mask and this row's don't meet (c0 is a multiple of 16):
                 // beside the MMAs
                 const uint4 mU = *reinterpret_cast<const uint4*>(tc.mU + c0 + f * kTcN + 8 * half);
                 const uint4 mm = make_uint4(mU.x & mL, mU.y & mL, mU.z & mL, mU.w & mL);
                 unsigned live = nc > 0 ? (1u << nc) - 1 : 0u;
                 if (tc_zero_half(mm.x) | tc_zero_half(mm.y) | tc_zero_half(mm.z) | tc_zero_half(mm.w)) {
-                    const unsigned apart = live & tc_zero_halves(mm);
-                    if (apart) upd_fma(cp, lda, A + (c0 + f * kTcN + 8 * half) * lda + k0, prw, apart);
-                    live &= ~apart;
+                    const unsigned apart = live & tc_apart(mU, nL);
+                    if (apart) live &= ~upd_fma(cp, lda, A + (c0 + f * kTcN + 8 * half) * lda + k0, prw, apart, eL, eU);
                 }
                 const bool ok = tc::mbar_wait(&tc.bar[a], ((tc.tiles + f) >> 1) & 1u, tc.deadline, tc.abort, tc.err);
                 if (!__all_sync(0xffffffffu, ok)) *tc.abort = 1;
                 tc::tc_fence_after();
                 cut_u(t + 1);                              // tile t - 1's slices have been read
                 const uint32_t ta = tc.tmem + ((uint32_t)((warp & 3) * 32) << 16) + a * kTcAcc + half * 8;
-                const short* eU = tc.eU + c0 + f * kTcN + 8 * half;
 #pragma unroll
                 for (int j4 = 0; j4 < 2; j4++) {
                     uint32_t g[kTcSlices][4];
