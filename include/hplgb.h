@@ -293,7 +293,9 @@ int lu_solve_backward(int64_t n, int64_t nrhs, const double* A, int64_t lda, con
  * copy; ws must hold solve_batched_workspace_size bytes) and launches nothing.
  * solve_batched_run (re)launches the planned work on `stream`: a queue reset
  * and one kernel, no host synchronisation, so it can be captured into a CUDA
- * graph and replayed; max_ctas <= 0 means one CTA per SM. solve_batched is
+ * graph and replayed; max_ctas <= 0 means as many CTAs as the SMs hold. Every
+ * run writes every system's info; one whose waits exceed opts->timeout_ns, and
+ * those that no CTA is left to take then, get HPL_ERR_TIMEOUT. solve_batched is
  * plan + run. hpl_batch_sizes draws the sizes of the batched workload,
  * n_s = 32 + (draw s of generator stream 2 mod 481), into a host array.
  */

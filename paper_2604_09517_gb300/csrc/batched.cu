@@ -31,6 +31,7 @@
 #include <utility>
 #include <vector>
 
+#include "batch_queue.cuh"
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -68,12 +69,13 @@ struct Sys {
 // mostly-FP32 one run side by side. The counters are cleared by every run.
 constexpr int kMaxSmSlots = 512;
 struct Header {
-    unsigned int counter[2];    // next index in list 0 / list 1
+    Queue queue;
     int count0;                 // systems in list 0
     int count;
     int max_iter;
     int nb_max;                 // widest panel of the plan (16 or 32)
     double tol;
+    long long timeout_ns;       // limit of a system's waits
     unsigned int sm_slot[kMaxSmSlots];   // CTAs started per SM (role by arrival)
 };
 
@@ -194,8 +196,8 @@ constexpr int kTcB = kTcSlices * kTcN * 16 * 2;      // 4 KB: a tile's U, two bu
 constexpr int kTcAcc = kTcSlices * kTcN;             // TMEM columns of an accumulator, two of them
 constexpr int kTcCols = 2 * kTcAcc;
 // Smaller updates take upd64. 304 systems of 64 / 96 / 128 / 512 with the line at 16,
-// 32, 64 and 96 rows (ms): 0.255, 0.261, 0.278, 0.278 / 0.443, 0.445, 0.462, 0.542 /
-// 0.655, 0.661, 0.672, 0.755 / 12.26, 12.29, 12.29, 12.32: 16 and 32 do not differ.
+// 32, 64 and 96 rows (ms): 0.257, 0.257, 0.276, 0.278 / 0.439, 0.443, 0.459, 0.542 /
+// 0.652, 0.655, 0.668, 0.751 / 11.94, 12.09, 11.98, 12.03: 16 and 32 do not differ.
 constexpr int kTcMinRows = 32;
 struct TcState {
     uint32_t tmem;
@@ -1168,6 +1170,7 @@ extern "C" int solve_batched_plan(int64_t count, const int64_t* n, double* const
     h.count0 = (int)count0;
     h.max_iter = o.max_iter;
     h.tol = o.tol;
+    h.timeout_ns = o.timeout_ns;
     h.nb_max = 16;
     for (int64_t s = 0; s < count; s++)
         if (!variant || variant[s] == 0) h.nb_max = bt::NBMAX;
@@ -1234,7 +1237,7 @@ extern "C" int solve_batched_run(void* ws, hpl_info* infos, int max_ctas, void* 
     const bool narrow = bt::planned_nb(ws) == 16 && bt::g_residency_mode == 0;
     const int per_sm = narrow ? 2 : 1;
     int grid = max_ctas > 0 ? std::min(max_ctas, per_sm * sms) : per_sm * sms;
-    HPL_CUDA_TRY(cudaMemsetAsync(H->counter, 0, sizeof(H->counter), s));
+    HPL_CUDA_TRY(cudaMemsetAsync(&H->queue, 0, sizeof(H->queue), s));
     HPL_CUDA_TRY(cudaMemsetAsync(H->sm_slot, 0, sizeof(H->sm_slot), s));
     if (narrow)
         bt::k_batched_run<16, 2><<<grid, bt::THREADS, bt::smem_bytes<16>(), s>>>(table, H, infos);
@@ -1294,34 +1297,26 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
                (short*)X + NMAX, (unsigned short*)X + 2 * NMAX, s_xk};
     const int pref = s_pref;
     const int lo[2] = {0, H->count0}, sz[2] = {H->count0, H->count - H->count0};
+    auto add = [](unsigned int* p, unsigned int v) { return atomicAdd(p, v); };
+    auto reset = [](hpl_info* info, int status) {
+        info->status = status;
+        info->iters = 0;
+        info->info = 0;
+        info->scaled_residual = 0.0;
+        info->inner_iters = 0;
+    };
     for (;;) {
-        if (threadIdx.x == 0) {
-            int idx = -1;
-            for (int q = 0; q < 2 && idx < 0; q++) {
-                const int l = pref ^ q;
-                if (sz[l] > 0 && (int)*(volatile unsigned int*)&H->counter[l] < sz[l]) {
-                    const int t = (int)atomicAdd(&H->counter[l], 1u);
-                    if (t < sz[l]) idx = lo[l] + t;
-                }
-            }
-            s_idx = idx;
-        }
+        if (threadIdx.x == 0) s_idx = queue_next(&H->queue, lo, sz, pref, add);
         __syncthreads();
         const int idx = s_idx;
         __syncthreads();
         if (idx < 0) break;
         const Sys S = table[idx];
         hpl_info* info = infos + S.pad;
-        if (threadIdx.x == 0) {
-            info->status = 0;
-            info->iters = 0;
-            info->info = 0;
-            info->scaled_residual = 0.0;
-            info->inner_iters = 0;
-        }
+        if (threadIdx.x == 0) reset(info, HPL_OK);
         __syncthreads();
         if (S.kind == 0) {
-            tc.deadline = globaltimer_ns() + (uint64_t)kDefaultTimeoutNs;
+            tc.deadline = globaltimer_ns() + (uint64_t)H->timeout_ns;
             bool ok;
             if constexpr (NBR == 16) {
                 ok = lu64<16>(S, P, Us, redk, redi, info, tc);
@@ -1342,6 +1337,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
         __syncthreads();
     }
     if (s_abort && threadIdx.x == 0) {
+        queue_give_up(&H->queue, lo, sz, gridDim.x, add,
+                      [&](int i) { reset(infos + table[i].pad, HPL_ERR_TIMEOUT); });
         // a wait gave up: the MMAs issued so far end (or have a second) before
         // TMEM is released
         __shared__ uint64_t s_drain;
