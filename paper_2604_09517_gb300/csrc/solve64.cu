@@ -624,7 +624,9 @@ static int solve_wave(int64_t n, const double* LU, int64_t lda, double* b, doubl
 // x_j for every block j solved before it, in sweep order, then substitute
 // inside the diagonal block (lane = row, warp = right-hand side, the solved
 // value passed by shuffle; the block's rows are scaled by the reciprocals of
-// its diagonal first, so a step of the substitution is one FMA). Solved blocks
+// its diagonal first, so a step of the substitution is one FMA; a block where
+// such a quotient leaves the range of normal numbers is solved unscaled, a
+// product and an FMA a step). Solved blocks
 // go to B; a counter per group and sweep (its front) says how many are there.
 //
 // What bounds it: FP64 issues 2 FMA per clock and SM, so n = 4096 with 64
@@ -636,11 +638,11 @@ static int solve_wave(int64_t n, const double* LU, int64_t lda, double* b, doubl
 // next tile of both is read into registers ahead of need; (d) 16 warps share
 // an SM, so the barriers of one CTA hide behind another's FMAs. The order of
 // additions into an entry does not depend on the schedule, so neither do the
-// bits. n = 4096 with 64 columns, plain and transposed solve together: 5.1 ms
+// bits. n = 4096 with 64 columns, plain and transposed solve together: 5.0 ms
 // (the FP64 rate allows 3.4), against 52 ms
 // with a diagonal and an update launch per 64 rows, one CTA on the diagonal;
-// with 2 columns a step of the chain costs 4.8 us. Each pass hands the front on
-// by hand_out's alternating words (5.2 ms with one word, which a pass that waits
+// with 2 columns a step of the chain costs 4.9 us. Each pass hands the front on
+// by hand_out's alternating words (one word, which was no faster, a pass that waits
 // could overwrite before the last warps had read it).
 //
 // Waits are bounded as in k_trsv_wave.
@@ -682,7 +684,9 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
     double* rhs = dinv + kMb;                         // [owned block][right-hand side][row], own thread only
     int* nj = (int*)(rhs + (size_t)R * T);            // [owned block] columns subtracted so far
     int* s_front = nj + R;                            // [2] thread 0's view of the front, alternating
+    int* s_plain = s_front + 2;                       // tag of the last block whose scaling is out of range
     int pass = 0;
+    if (t == 0) *s_plain = 0;
     const uint64_t deadline = globaltimer_ns() + (uint64_t)timeout_ns;
     const bool live = warp < ncol;
     double* bcol = B + (c0 + (live ? warp : 0)) * ldb;
@@ -722,16 +726,27 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
             const int64_t row = (int64_t)j * kMb + lane;
             return live && row < n ? __ldcg(bcol + row) : 0.0;
         };
-        // the diagonal block of row block q, rows scaled by the reciprocals
-        auto load_diag = [&](int q) {
+        // the diagonal block of the sweep's owned block k, rows scaled by the
+        // reciprocals; a quotient out of range leaves the block's tag in *s_plain
+        auto tag = [&](int k) { return sweep * R + k + 1; };
+        auto load_diag = [&](int k) {
+            const int q = qk(k);
             const int64_t r = (int64_t)q * kMb + lane;
             if (warp == 0) dinv[lane] = !unit && r < n ? 1.0 / LU[r * lda + r] : 1.0;
             double v[E];
             load_tile(q, q, v);
             __syncthreads();
             if (!unit) {
+                bool out = false;
 #pragma unroll
-                for (int e = 0; e < E; e++) v[e] *= dinv[trans ? warp + W * e : lane];
+                for (int e = 0; e < E; e++) {
+                    const double d = v[e] * dinv[trans ? warp + W * e : lane];
+                    const unsigned x = (unsigned)__double2hiint(d) >> 20 & 0x7ffu;
+                    out = out || x == 0x7ffu ||
+                          (x == 0 && ((unsigned)__double2hiint(v[e]) << 1 | (unsigned)__double2loint(v[e])) != 0);
+                    v[e] = d;
+                }
+                if (out) *s_plain = tag(k);
             }
             store_tile(dtile, v);
         };
@@ -741,7 +756,7 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
         int ks = R > 1 ? 1 : -1, js = 0;               // the slack's block and column
         bool xpv = false, xsv = false;                 // x of the column read ahead
         double pn[E], sn[E], xp = 0.0, xn = 0.0;
-        load_diag(qk(0));
+        load_diag(0);
         if (pos(0) > 0) load_tile(qk(0), qs(0), pn);
         if (ks > 0) load_tile(qk(ks), qs(0), sn);
         double acc = rhs[(size_t)slot(0) * T + t];
@@ -762,15 +777,30 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
         for (;;) {
             if (jp == pos(kp)) {
                 // all columns subtracted: substitution in the diagonal block
-                if (!unit) acc *= dinv[lane];
-                if (live) {
-#pragma unroll
+                if (*s_plain == tag(kp)) {             // solved with the block as it is
+                    double v[E];
+                    load_tile(qk(kp), qk(kp), v);
+                    store_tile(dtile, v);
+                    __syncthreads();
+#pragma unroll 1
                     for (int s2 = 0; s2 < kMb; s2++) {
                         const int j = fwd ? s2 : kMb - 1 - s2;
-                        const double xj = __shfl_sync(0xffffffffu, acc, j);
-                        const double d = dtile[j * kMbLd + lane];
-                        if (fwd ? lane > j : lane < j) acc = fma(-d, xj, acc);
+                        const double xj = __shfl_sync(0xffffffffu, acc * dinv[lane], j);
+                        if (lane == j) acc = xj;
+                        else if (fwd ? lane > j : lane < j) acc = fma(-dtile[j * kMbLd + lane], xj, acc);
                     }
+                } else {
+                    if (!unit) acc *= dinv[lane];
+                    if (live)
+#pragma unroll
+                        for (int s2 = 0; s2 < kMb; s2++) {
+                            const int j = fwd ? s2 : kMb - 1 - s2;
+                            const double xj = __shfl_sync(0xffffffffu, acc, j);
+                            const double d = dtile[j * kMbLd + lane];
+                            if (fwd ? lane > j : lane < j) acc = fma(-d, xj, acc);
+                        }
+                }
+                if (live) {
                     const int64_t row = (int64_t)qk(kp) * kMb + lane;
                     if (row < n) __stcg(bcol + row, acc);
                 }
@@ -786,7 +816,7 @@ k_trsm_wave(int64_t n, int64_t nrhs, const double* __restrict__ LU, int64_t lda,
                 acc = rhs[(size_t)slot(kp) * T + t];
                 if (jp < pos(kp)) load_tile(qk(kp), qs(jp), pn);
                 xpv = false;
-                load_diag(qk(kp));
+                load_diag(kp);
                 if (ks == kp) {
                     ks = kp + 1 < R ? kp + 1 : -1;
                     if (ks > 0) {
@@ -911,7 +941,7 @@ static int solve_multi(int64_t n, int64_t nrhs, const double* LU, int64_t lda, d
                        int* flags, int64_t nflags, int* abort_flag, hpl_info* info, cudaStream_t s) {
     const size_t limit = wave_smem_limit();
     const int64_t nblk = (n + kMb - 1) / kMb;
-    auto bytes = [](int64_t R) { return msolve_smem_doubles(W, (int)R) * sizeof(double) + (size_t)(R + 2) * sizeof(int); };
+    auto bytes = [](int64_t R) { return msolve_smem_doubles(W, (int)R) * sizeof(double) + (size_t)(R + 3) * sizeof(int); };
     // blocks a CTA may own with 16 / W CTAs on an SM (a KB of each is reserved)
     const size_t share = limit / (16 / W) - 1024;
     if (share < bytes(1) || n > (int64_t)1 << 30) return -1;

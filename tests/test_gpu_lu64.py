@@ -532,6 +532,34 @@ def test_lu_solve_several_columns_repeats_its_bits(hpl, nrhs, trans):
         hpl.lu_config(hpl.LU_SOLVE_WAVE_GRID, 0)
 
 
+@pytest.mark.parametrize("trans", [0, 1])
+@pytest.mark.parametrize("e", [600, -600])
+def test_lu_solve_several_columns_far_from_the_diagonal(hpl, e, trans):
+    """Rows of a triangle whose entries over the diagonal's are beyond 2^1023 or
+    below 2^-1074, with solutions in range: powers of two, so every digit is
+    right. The other row blocks' columns are untouched."""
+    import torch
+    n, nrhs = 130, 3
+    A = torch.eye(n, dtype=torch.float64)
+    B = torch.ones(n, nrhs, dtype=torch.float64)
+    want = B.clone()
+    f = 1 if e > 0 else -1
+    for p in (0, 30, 62, 96):
+        q = p + 1
+        top, low = (q, p) if trans else (p, q)      # the row solved second, the one first
+        A[p, q] = 2.0 ** (500 * f)
+        A[top, top] = 2.0 ** -e
+        B[low], B[top] = 2.0 ** (-700 * f), 3 * 2.0 ** (-200 * f)
+        want[low], want[top] = 2.0 ** (-700 * f), 2.0 ** (1 - 200 * f + e)
+    LU, X = A.t().contiguous().t().cuda(), B.t().contiguous().t().cuda()
+    ipiv = torch.arange(n, dtype=torch.int32, device="cuda")
+    info = hpl.Info()
+    hpl.lu_solve(LU, ipiv, X, trans=trans, info=info)
+    torch.cuda.synchronize()
+    assert info.read()["status"] == 0
+    assert torch.equal(X.cpu(), want)
+
+
 @pytest.mark.parametrize("kind", ["uniform", "ties"])
 @pytest.mark.parametrize("n,nb,la", [(2, 64, 0), (31, 32, 0), (33, 64, 1), (65, 64, 0), (129, 40, 1), (513, 64, 0),
                                      (1100, 256, 1), (1700, 96, 1), (2200, 256, 1), (4300, 128, 1)])
