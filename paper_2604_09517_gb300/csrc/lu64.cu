@@ -773,21 +773,20 @@ constexpr int kTrsmCols = 16;
 
 // kk <= 64: L11 staged in shared memory once (the loop above re-reads a
 // column of L from L2 at every step, which at this size is latency, not
-// work), COLS columns of B per CTA, loads and stores coalesced along rows.
-template <int COLS>
+// work), 16 columns of B per CTA, loads and stores coalesced along rows.
 __global__ void __launch_bounds__(256) k_trsm_lunit_small(double* __restrict__ A, int64_t lda, int64_t r0, int kk,
                                                           int64_t cb, int64_t ce) {
-    constexpr int G = 256 / COLS;
+    constexpr int G = 256 / kTrsmCols;
     __shared__ double Ls[64][65];
-    __shared__ double xs[64][COLS];
-    const int c = threadIdx.x % COLS, g = threadIdx.x / COLS;
-    const int64_t cbase = cb + (int64_t)blockIdx.x * COLS;
-    const int ncol = (int)min((int64_t)COLS, ce - cbase);
+    __shared__ double xs[64][kTrsmCols];
+    const int c = threadIdx.x % kTrsmCols, g = threadIdx.x / kTrsmCols;
+    const int64_t cbase = cb + (int64_t)blockIdx.x * kTrsmCols;
+    const int ncol = (int)min((int64_t)kTrsmCols, ce - cbase);
     for (int idx = threadIdx.x; idx < kk * kk; idx += 256) {
         const int j = idx / kk, i = idx - j * kk;
         if (i > j) Ls[i][j] = A[(r0 + j) * lda + r0 + i];
     }
-    for (int idx = threadIdx.x; idx < kk * COLS; idx += 256) {
+    for (int idx = threadIdx.x; idx < kk * kTrsmCols; idx += 256) {
         const int cc = idx / kk, i = idx - cc * kk;
         xs[i][cc] = cc < ncol ? A[(cbase + cc) * lda + r0 + i] : 0.0;
     }
@@ -1225,7 +1224,7 @@ static int launch_trsm(double* A, int64_t lda, int64_t r0, int kk, int64_t cb, i
     if (ce <= cb || kk <= 1) return HPL_OK;
     if (kk <= 64) {
         if ((ce - cb) / 16 >= kNumSMsGB300) {
-            k_trsm_lunit_small<16><<<(unsigned)((ce - cb + 15) / 16), 256, 0, s>>>(A, lda, r0, kk, cb, ce);
+            k_trsm_lunit_small<<<(unsigned)((ce - cb + 15) / 16), 256, 0, s>>>(A, lda, r0, kk, cb, ce);
         } else {
             // as few columns per CTA as keep the grid near one CTA per SM
             const int64_t nx = ce - cb;
