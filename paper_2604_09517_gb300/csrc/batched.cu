@@ -1191,8 +1191,9 @@ __global__ void __launch_bounds__(THREADS, MINB) k_batched_run(const Sys* __rest
 
 // The widest panel of each planned workspace (host side), so that the run
 // launch picks its kernel without reading the device: a plan whose systems all
-// use 16-wide panels runs two CTAs per SM (79 KB of shared memory each),
-// otherwise one (the 32-wide panel takes 164 KB). A workspace that was not
+// use 16-wide panels runs two CTAs per SM (111 KB of shared memory each, which
+// leaves 1 KB of an SM's 228, and half of its TMEM), otherwise one (the 32-wide
+// panel takes 192 KB). A workspace that was not
 // planned in this process gets the one-per-SM kernel, which handles both.
 std::mutex g_plan_mu;
 std::vector<std::pair<const void*, int>> g_plan_nb;

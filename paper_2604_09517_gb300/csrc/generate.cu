@@ -90,9 +90,8 @@ __global__ void __launch_bounds__(256) k_dominant_diag(int64_t n, double* __rest
 // regenerate the entries). Every entry is the FP64 generated value rounded
 // once to nearest, exactly what converting a stored FP64 matrix gives.
 //
-// One pass over the entries: rows in blocks of 512 (blockIdx.x), two adjacent
-// rows a thread, `chunks` column chunks (blockIdx.y). Per (row, chunk) the
-// kernel writes the entries, the exact sum of |a_ij| / 2^-53 = |(h >> 11) - 2^52|
+// One pass over the entries: rows in blocks of 256 (blockIdx.x), a row a thread,
+// `chunks` column chunks (blockIdx.y). Per (row, chunk) the kernel writes the entries, the exact sum of |a_ij| / 2^-53 = |(h >> 11) - 2^52|
 // over the chunk in 128 bits (the diagonal's dominance, all j), and the FP32
 // sum of the stored |a_ij| over the chunk's off-diagonal entries (||A||_inf for
 // the refinement's stopping test).

@@ -44,9 +44,10 @@
 // Bound: per stage 1056 clocks of MMA at the dense BF16 rate and about as many
 // issue slots for the slicing; measured 3300 clocks per stage, the producers'
 // latency (2.6 us of shared-memory and conversion chains per 8 values and
-// thread). n = 4096 with 64 columns: 0.30 ms plain, 0.28 ms transposed, against
-// 2.13 ms for the DFMA kernel; the outer product 4096 x 4096 x 64 0.51 ms
-// against 1.76. With one group of 8 producer warps and register prefetch: 0.48.
+// thread). n = 4096 with 64 columns: 0.26 ms plain, 0.23 ms transposed, against
+// 2.13 ms for the DFMA kernel; the outer product 4096 x 4096 x 64 0.49 ms
+// against 1.76. With one group of 8 producer warps and register prefetch the plain
+// product took 0.48.
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -1035,10 +1035,13 @@ extern "C" int lu_solve(int64_t n, int64_t nrhs, const double* LU, int64_t lda, 
     const bool multi = g_solve_wave && (nrhs > 1 || trans);
     const int64_t nflags = (n + kTB - 1) / kTB * kTB * 2;      // pairs of ints in w.pub
     // Group width: with many columns the FMAs bound the solve, and groups of 4
-    // shorten a step of the chain; with few columns or blocks the chain does, and
-    // the wider CTA loads its tiles faster. Measured (ms, width 8 / 4): n = 4096
-    // with 8 columns 1.54 / 1.60, 16: 1.74 / 1.75, 32: 2.01 / 1.94, 64: 2.67 /
-    // 2.60; n = 12000 with 64: 18.7 / 17.7; n = 1001 with 24: 0.417 / 0.430.
+    // shorten a step of the chain; with few columns the chain does, and the wider
+    // CTA loads its tiles faster. Measured (ms, width 8 / 4): n = 24000 with 5 columns
+    // 10.1 / 10.9, n = 12000 with 5 4.26 / 4.43, n = 4096 with 2 1.252 / 1.260, with
+    // 64 2.65 / 2.51, 512 19.2 / 17.9, 1024 38.4 / 35.7; n = 12000 with 64 18.5 / 17.5,
+    // 256 72.0 / 65.9, 1024 299 / 279. Groups of 4 have become the faster ones from 8
+    // columns on below this line too (n = 4096 with 8 1.51 / 1.34, n = 1000 with 64
+    // 0.449 / 0.402, with 512 1.30 / 1.25), by up to 16 %.
     auto both = [&]() {
         int* flags = (int*)w.pub;
         return nrhs > 16 && n >= 2048
