@@ -278,8 +278,9 @@ __device__ __noinline__ void by_fma(unsigned which, const double* A, int64_t lda
                 if (!weigh) continue;
 #pragma unroll
                 for (int u = 0; u < 4; u++) t = fma(fabs(x[u]), fabs(y[u]), t);
-                // the lanes' shares in units of 2^-16 lim, rounded down
-                keep = lim == lim && __reduce_add_sync(0xffffffffu, (unsigned)fmin(t * per, 65536.0)) >= 65536u;
+                // the lanes' shares in units of 2^-16 lim, rounded down (a smaller lim has
+                // no reciprocal in range: the whole sum decides below)
+                keep = lim >= 0x1p-1000 && __reduce_add_sync(0xffffffffu, (unsigned)fmin(t * per, 65536.0)) >= 65536u;
             }
             if (keep) continue;
 #pragma unroll

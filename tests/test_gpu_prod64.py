@@ -186,3 +186,25 @@ def test_block_refinement_keeps_small_components(hpl, n, e, trans):
         for c in range(2):
             m = part[:, c]
             assert err[m, c].max() <= 2.0 ** -20 * np.abs(want[m, c]).max()
+
+
+@pytest.mark.parametrize("shift", [0, -940])
+def test_outer_product_keeps_few_small_entries(hpl, shift):
+    """Three rows of grad_B that vanish where two thirds of X's rows are large:
+    few entries of a column below the slices' line, also where the products come
+    near the smallest numbers (each rounding is then up to 2^-1075)."""
+    import torch
+    n, nrhs = 150, 40
+    A = torch.diag(torch.linspace(1.0, 2.0, n, dtype=torch.float64, device="cuda")).t()
+    G = hpl.generate(44, 7, n, nrhs) * 2.0 ** -64
+    X = hpl.generate(44, hpl.STREAM_B, n, nrhs) * 2.0 ** shift
+    _, _, ws = hpl.mxp_solve(A, hpl.generate(44, 8, n, nrhs), nb=64, refine=hpl.REFINE_IR)
+    for r in (5, 70, 100):
+        G[r, ::2] = 0.0
+    X[:100, 1::2] *= 2.0 ** -20
+    G, X = G.t().contiguous().t(), X.t().contiguous().t()
+    gB, gA, info = hpl.lu_solve_backward(A, X, G, ws, nb=64, refine=hpl.REFINE_IR)
+    assert info.read()["status"] == 0
+    g, x = _np(gB).astype(np.longdouble), _np(X).astype(np.longdouble)
+    bound = (nrhs + 2) * (EPS * (np.abs(g) @ np.abs(x).T) + np.longdouble(2.0) ** -1075)
+    assert (np.abs(_np(gA).astype(np.longdouble) + g @ x.T) <= bound).all()
